@@ -123,6 +123,16 @@ struct pic_ctx {
     PersistCfg pcfg;
     cudaGraphExec_t persist_graph = nullptr;
     bool persist_direct = false;     // the launch could not be captured: launched directly
+    // grouped steps (event_pass 0): their configuration, the counts of the
+    // record lists, removals per step, block sums, results, barriers and the
+    // tail blocks' shares
+    GroupCfg gc;
+    GroupArgs ga{};
+    uint16_t *d_gcnt = nullptr;
+    uint32_t *d_gabs = nullptr, *d_gsum = nullptr;
+    GroupRes *d_gres = nullptr;
+    unsigned int *d_gbar = nullptr;
+    int4 *d_gblk = nullptr;
     // kernel timing (pic_profile)
     bool profiling = false;
     std::vector<cudaEvent_t> ev_pool;
@@ -381,6 +391,8 @@ void free_all(pic_ctx *c)
     release(c->d_w[0]); release(c->d_w[1]); release(c->d_wcell); release(c->d_wbin);
     release(c->d_kthr); release(c->d_nhw); release(c->d_bdw); release(c->d_Jw); release(c->d_hnow_w);
     release(c->d_ctl);
+    release(c->d_gcnt); release(c->d_gabs); release(c->d_gsum); release(c->d_gres); release(c->d_gbar);
+    release(c->d_gblk);
     Replay &r = c->rp;
     for (int b = 0; b < 2; ++b) {
         r.pk[b] = nullptr;                      // inside r.mu[b]
@@ -711,9 +723,66 @@ pic_status pic_init(pic_ctx **out, const pic_params *p, const pic_stack_desc *st
     a.qcnt = c->d_qcnt;
     a.fspawn = c->d_fspawn;
 
+    // grouped steps, where their shared memory fits
+    e = configure_group(a, c->total_slots, &c->gc);
+    std::vector<int4> blk;
+    if (e == cudaSuccess && c->gc.ok) {
+        GroupArgs &g = c->ga;
+        const int gt = c->gc.grid_tail;
+        g.cnt_n = c->total_slots / GROUP_SUB_MIN + 1;
+        e = dalloc(&c->d_gcnt, (size_t)GROUP_OPEN * g.cnt_n);
+        if (e == cudaSuccess) e = dalloc(&c->d_gabs, (size_t)n_stacks * GROUP_MAX);
+        if (e == cudaSuccess) e = dalloc(&c->d_gsum, (size_t)2 * GROUP_OPEN * gt);
+        if (e == cudaSuccess) e = dalloc(&c->d_gres, n_stacks);
+        if (e == cudaSuccess) e = dalloc(&c->d_gbar, (size_t)2 * n_stacks);
+        if (e == cudaSuccess) e = dalloc(&c->d_gblk, gt);
+        // every stack one block, the others by capacity (the rest to the largest)
+        std::vector<int> nb(n_stacks, 1);
+        int left = gt - n_stacks, big = 0;
+        const int spare = left;
+        for (int s = 0; s < n_stacks; ++s) {
+            const int add = (int)((double)spare * (double)c->hs[s].cap_round / (double)std::max<int64_t>(c->total_slots, 1));
+            nb[s] += std::min(add, left);
+            left -= std::min(add, left);
+            if (c->hs[s].cap_round > c->hs[big].cap_round) big = s;
+        }
+        nb[big] += left;
+        for (int s = 0; s < n_stacks; ++s) {
+            const int first = (int)blk.size();
+            for (int i = 0; i < nb[s]; ++i) blk.push_back(make_int4(s, i, nb[s], first));
+        }
+        // the lists of the four steps: one 8-byte record per slot and step, in
+        // the buffers of the single steps' staged and queued records
+        g.list[0] = reinterpret_cast<uint2 *>(c->d_stage);
+        g.list[1] = reinterpret_cast<uint2 *>(c->d_qrec);
+        g.list_n = c->total_slots;
+        g.cnt = c->d_gcnt;
+        g.abs = c->d_gabs;
+        g.bsum = c->d_gsum;
+        g.tsum = c->d_gsum + (size_t)GROUP_OPEN * gt;
+        g.res = c->d_gres;
+        g.bar = c->d_gbar;
+        g.blk = c->d_gblk;
+        g.sub = 128 * c->gc.quads;
+        g.nd = c->gc.nd;
+        g.nj = c->gc.nj;
+    }
+    if (e != cudaSuccess) {
+        g_init_error = std::string("grouped steps: ") + cudaGetErrorString(e);
+        free_all(c);
+        delete c;
+        cudaGetLastError();
+        return PIC_ERR_ALLOC;
+    }
+
     cudaStream_t st = c->stream;
     DevCtl ctl{};
     ctl.epoch = 1u;
+    if (c->gc.ok) {
+        e = cudaMemsetAsync(c->d_gabs, 0, sizeof(uint32_t) * (size_t)n_stacks * GROUP_MAX, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->d_gbar, 0, sizeof(unsigned int) * 2 * (size_t)n_stacks, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_gblk, blk.data(), sizeof(int4) * blk.size(), cudaMemcpyHostToDevice, st);
+    }
     std::vector<DevCounters> cnt(n_stacks);
     std::memset(cnt.data(), 0, sizeof(DevCounters) * n_stacks);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_stacks, c->ds.data(), sizeof(DevStack) * n_stacks, cudaMemcpyHostToDevice, st);
@@ -890,6 +959,61 @@ bool any_source(const pic_ctx *c, int s0, int n)
     return false;
 }
 
+// Whether the context's steps run in groups (pic_group.cu).
+bool grouped(const pic_ctx *c) { return c->gc.ok && c->p.event_pass == 0; }
+
+// First step after s at which a range of grouped steps must end: the next
+// compaction, the next density step unless the densities are deposited inside
+// the groups, and what one closed group may hold.
+int range_end(const pic_ctx *c, int s)
+{
+    const int ce = c->p.compact_every, me = c->p.moment_every;
+    int e = std::min((s / ce + 1) * ce, s + GROUP_MAX);
+    if (!c->gc.dep) e = std::min(e, (s / me + 1) * me);
+    return e;
+}
+
+// Steps [s, e) in groups, then what is due at their end.  Every group's
+// launches are issued for the case that the groups before it were open; one
+// that a closed group has run past leaves at once.  `base`: s and e count from
+// *base (graph capture; src: a source in the period), else from 0.
+cudaError_t enqueue_range(pic_ctx *c, const Args &a0, int s, int e, const unsigned int *base, bool src,
+                          cudaStream_t st, int64_t &launches)
+{
+    const bool det = (c->p.flags & PIC_F_DETERMINISTIC) != 0;
+    const GroupCfg &gc = c->gc;
+    Args a = a0;
+    a.step_dev = &c->d_ctl->step;
+    a.bump_step = 0;
+    GroupArgs g = c->ga;
+    g.base = base;
+    g.end = e;
+    cudaError_t r = cudaSuccess;
+    for (int o = s; o < e && r == cudaSuccess; o += g.m) {
+        g.off = o;
+        g.m = std::min(gc.m, e - o);
+        g.no_src = base ? !src : !any_source(c, o, e - o);
+        r = timed(c, gc.dep ? 2 : 1, [&] { return launch_group(a, g, gc, det, st); });
+        if (r == cudaSuccess) r = timed(c, 4, [&] { return launch_tail(a, g, gc, det, st); });
+        launches += 2;
+    }
+    if (r == cudaSuccess && e % c->p.moment_every == 0) {
+        if (!gc.dep) {
+            r = timed(c, 2, [&] { return launch_dens(a, gc, st); });
+            ++launches;
+        }
+        if (r == cudaSuccess && (c->p.flags & PIC_F_WEIGHTS)) {
+            r = timed(c, 9, [&] { return launch_wdep(a, c->lc, st); });
+            ++launches;
+        }
+    }
+    if (r == cudaSuccess && e % c->p.compact_every == 0) {
+        r = timed(c, 3, [&] { return launch_compact(a, c->lc, st); });
+        ++launches;
+    }
+    return r;
+}
+
 // Capture one period of steps (starting at a step that is a multiple of the
 // period) into a graph; with_source: the source kernels of every half step.
 cudaError_t capture_period(pic_ctx *c, int which)
@@ -905,8 +1029,18 @@ cudaError_t capture_period(pic_ctx *c, int which)
     int64_t n = 0;
     cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
-    for (int i = 0; i < c->period && e == cudaSuccess; ++i)
-        e = enqueue_step(c, a, i, src, src, true, c->cap_stream, n);
+    if (grouped(c)) {
+        e = launch_mark_base(c->d_ctl, c->cap_stream);
+        ++n;
+        for (int i = 0; i < c->period && e == cudaSuccess;) {
+            const int i1 = std::min(range_end(c, i), c->period);
+            e = enqueue_range(c, a, i, i1, &c->d_ctl->base, src, c->cap_stream, n);
+            i = i1;
+        }
+    } else {
+        for (int i = 0; i < c->period && e == cudaSuccess; ++i)
+            e = enqueue_step(c, a, i, src, src, true, c->cap_stream, n);
+    }
     const cudaError_t e2 = cudaStreamEndCapture(c->cap_stream, &g);
     if (e == cudaSuccess) e = e2;
     if (e == cudaSuccess) e = cudaGraphInstantiate(&c->period_graph[which], g, 0);
@@ -1043,6 +1177,19 @@ pic_status pic_step(pic_ctx *c, int n_steps)
             c->launches += c->period_launches[which];
             c->step = s + c->period;
             left -= c->period;
+            continue;
+        }
+        if (grouped(c)) {
+            const int s1 = std::min(range_end(c, s), s + left);
+            if (!c->dev_step_valid) {
+                e = launch_set_step(c->d_ctl, (unsigned int)s, c->stream);
+                c->launches += 1;
+            }
+            if (e == cudaSuccess) e = enqueue_range(c, c->args, s, s1, nullptr, false, c->stream, c->launches);
+            if (e != cudaSuccess) return cuda_fail(c, e, "pic_step launch");
+            c->dev_step_valid = true;
+            c->step = s1;
+            left -= s1 - s;
             continue;
         }
         bool inj0 = false, inj1 = false;
@@ -1859,11 +2006,17 @@ pic_status pic_autotune(pic_ctx *c, int trial_steps, pic_tune_entry *entries, in
     // the fused form exists for one stack and eight consumer warps, with at
     // most PIC_EV_MIN_BLOCKS blocks per SM
     const bool fusable = c->n_stacks == 1;
+    // grouped steps do not depend on the other options: one ring depth and
+    // deposit mode of them are tried
+    const bool grp = c->gc.ok;
     for (int hm = 0; hm <= (dep_in_trial ? 1 : 0); ++hm)
         for (int nw : {8, 4})
-            for (int ev = (nw == 8 && fusable ? 0 : 1); ev <= 1; ++ev)
+            for (int ev = (nw == 8 && (fusable || grp) ? 0 : 1); ev <= 1; ++ev)
                 for (int bps = 1; bps <= (ev == 0 ? 3 : nw == 4 ? 8 : 6); ++bps)
-                    for (int ring : {2, 3, 4, 6, 8}) cands.push_back({bps, ring, hm, nw, ev});
+                    for (int ring : {2, 3, 4, 6, 8}) {
+                        if (ev == 0 && grp && (ring != 2 || hm != 0)) continue;
+                        cands.push_back({bps, ring, hm, nw, ev});
+                    }
     if ((int64_t)c->step + (int64_t)trial_steps * (int64_t)cands.size() > c->p.n_steps_max)
         return fail(c, PIC_ERR_ARG, "pic_autotune: not enough steps left for the trials");
     const int use_graph = c->p.use_graph;
@@ -1906,15 +2059,21 @@ pic_status pic_autotune(pic_ctx *c, int trial_steps, pic_tune_entry *entries, in
         if (gmax > c->n_status || lc.ring_fast != k.ring || lc.grid_fast != sms * k.bps ||
             lc.grid_fast_dep == 0)
             continue;
-        if (k.ev == 0 && (lc.grid_fused != sms * k.bps || lc.ring_fused != k.ring)) continue;
+        if (k.ev == 0 && fusable && (lc.grid_fused != sms * k.bps || lc.ring_fused != k.ring)) continue;
         c->lc = lc;
         c->p.hist_mode = k.hm;
+        c->p.event_pass = k.ev;
         uint64_t ps0 = 0, ps1 = 0;
         e = steps_done(ps0);
         if (e == cudaSuccess) e = cudaEventRecord(ev[0], c->stream);
         if (e != cudaSuccess) break;
         const pic_status st = pic_step(c, trial_steps);
-        if (st != PIC_OK) { c->lc = keep; c->p = keep_p; c->p.use_graph = use_graph; return st; }
+        if (st != PIC_OK) {
+            c->lc = keep;
+            c->p = keep_p;
+            c->p.use_graph = use_graph;
+            return st;
+        }
         e = cudaEventRecord(ev[1], c->stream);
         if (e == cudaSuccess) e = steps_done(ps1);
         float ms = 0.f;

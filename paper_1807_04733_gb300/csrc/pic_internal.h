@@ -105,6 +105,7 @@ struct DevCtl {
     unsigned int step;       // time step of graph-replayed steps
     unsigned int bar_count;  // grid barrier of the persistent kernel: arrivals,
     unsigned int bar_gen;    //   and its generation
+    unsigned int base;       // first step of the graph being replayed (grouped steps)
 };
 
 struct Args {            // everything a kernel needs, passed by value
@@ -195,6 +196,42 @@ struct Args {            // everything a kernel needs, passed by value
     long long *v_hist;
 };
 
+// Groups of time steps run in one pass over memory (pic_group.cu).
+constexpr int GROUP_OPEN = 4;    // most steps of a group that may create secondaries
+constexpr int GROUP_MAX = 64;    // most steps of a closed group
+constexpr int GROUP_SUB_MIN = 256;   // fewest slots of a warp's sub-tile
+
+struct GroupRes {                // a stack's counters after a group (published by its first block)
+    unsigned long long n_slots, next_id, steps0, live0;
+};
+
+struct GroupArgs {
+    int off, end;                // the group's first step; the range it may run through
+    int m;                       // steps of an open group
+    int no_src;                  // no source carriers in [off, end)
+    const unsigned int *base;    // off and end count from *base (graph replay); null: from 0
+    // new secondaries (depth, k | layer | gen | position) of step j of the
+    // group: list_n entries at list[j / 2] + (j % 2) list_n
+    uint2 *list[2];
+    long long list_n;
+    uint16_t *cnt;               // [GROUP_OPEN][cnt_n] secondaries per sub-tile
+    long long cnt_n;
+    uint32_t *abs;               // [n_stacks][GROUP_MAX] carriers removed per step
+    uint32_t *bsum, *tsum;       // [GROUP_OPEN][tail blocks] secondaries per block
+    GroupRes *res;               // [n_stacks]
+    unsigned int *bar;           // [n_stacks][2] barrier of a stack's tail blocks
+    const int4 *blk;             // per tail block: stack, index in it, the stack's blocks, the first
+    int sub;                     // slots per sub-tile
+    int nd, nj;                  // density and removal windows held in shared memory
+};
+
+struct GroupCfg {
+    bool ok = false, dep = false;    // dep: densities deposited inside the group
+    int m = 0, quads = 0, warps = 0, nd = 0, nj = 0;
+    int grid = 0, grid_tail = 0, grid_dens = 0;
+    size_t smem = 0, smem_tail = 0, smem_dens = 0;
+};
+
 // reason of the last failure of a call without a context (pic_capi.cu);
 // returned by pic_last_error(NULL)
 void pic_set_static_error(const char *msg);
@@ -260,6 +297,17 @@ struct PersistCfg {
 cudaError_t configure_persistent(const Args &a, bool det, PersistCfg *pc);
 cudaError_t launch_persistent(const Args &a, const PersistCfg &pc, bool det, int n_steps,
                               cudaStream_t s);
+
+// grouped steps (pic_group.cu): the pass over the slots present at the group's
+// start, then the new carriers of every step of it; the densities of a
+// finished window where they are not deposited inside the group
+cudaError_t configure_group(const Args &a, long long slots, GroupCfg *gc);
+cudaError_t launch_group(const Args &a, const GroupArgs &g, const GroupCfg &gc, bool det,
+                         cudaStream_t s);
+cudaError_t launch_tail(const Args &a, const GroupArgs &g, const GroupCfg &gc, bool det,
+                        cudaStream_t s);
+cudaError_t launch_dens(const Args &a, const GroupCfg &gc, cudaStream_t s);
+cudaError_t launch_mark_base(DevCtl *ctl, cudaStream_t s);
 
 // adjoint replay (pic_adjoint.cu); pass = 1 or 2
 cudaError_t configure_adjoint(const Args &a, int pass, LaunchCfg *cfg);

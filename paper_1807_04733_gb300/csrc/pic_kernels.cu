@@ -670,7 +670,7 @@ cudaError_t launch_inject(const Args &a, const LaunchCfg &c, int half, bool depo
     return cudaGetLastError();
 }
 
-__global__ void k_set_step(DevCtl *ctl, unsigned int step) { ctl->step = step; }
+__global__ void k_set_step(DevCtl *ctl, unsigned int step) { ctl->step = ctl->base = step; }
 
 cudaError_t launch_set_step(DevCtl *ctl, unsigned int step, cudaStream_t s)
 {
