@@ -37,7 +37,7 @@ namespace pic {
 namespace {
 
 #ifndef PIC_GROUP_UNROLL
-#define PIC_GROUP_UNROLL 2
+#define PIC_GROUP_UNROLL 4
 #endif
 #ifndef PIC_GROUP_GW
 #define PIC_GROUP_GW 16
@@ -439,72 +439,53 @@ __global__ void __launch_bounds__(32 * GW_MAX, 1) k_group(const Args a, const Gr
                     int k = (int)(pk & 0xFFu), layer = (int)((pk >> 9) & 0xFu);
                     const int sg = (int)((pk >> 8) & 1u);
                     FastEnt e = s_ent[(((layer * 2 + sg) << a.kb) + k)];
-                    uint32_t xs;
-                    // what the sweep only suspected: the boundary and the test
-                    bool bnd, ev;
+                    // What the sweep suspected, settled: the first boundary of
+                    // the step, if any, and the test.  The word that comes next
+                    // is known but for a carrier that scatters before it meets
+                    // its boundary (it draws again), so both Philox calls run
+                    // side by side.
+                    bool dead = false, second, pend = false;
+                    float tau = half, zb;
+                    int hit = 0;
+                    uint32_t xs, sub_;
+                    uint4 r;
+                    bool up, ev;
                     {
-                        const uint4 x = philox_test((uint32_t)slot >> 2, tk, a);
-                        xs = (slot & 2) ? ((slot & 1) ? x.w : x.z) : ((slot & 1) ? x.y : x.x);
                         const float w = __fmul_rn(e.v, mu);
                         z = w < 0.f ? -z : z;
-                        const float z2 = fly<DET>(fly<DET>(z, w, half), w, half);
-                        bnd = act && (z2 > e.hi || z2 < e.lo);
-                        ev = bnd || (act && xs < e.P);
-                        if (!ev) z = z2;
-                    }
-                    n_event += (uint32_t)__popc(__ballot_sync(0xffffffffu, ev));
-                    bool dead = false, done = !ev, second = false;
-                    float tau = half;
-                    int hit = 0;
-                    uint2 srec = make_uint2(0u, 0u);
-                    // a lane flies until it needs a random word or is done;
-                    // one Philox call serves every lane that needs one
-#pragma unroll 1
-                    while (__any_sync(0xffffffffu, !done)) {
-                        uint32_t sub_ = 0;
-                        bool up = false;
-                        if (!done) {
-#pragma unroll 1
-                            for (;;) {
-                                const float w = __fmul_rn(e.v, mu);
-                                const float z1 = fly<DET>(z, w, tau);
-                                up = mu > 0.f;
-                                const float zb = up ? e.hi : e.lo;
-                                const bool cross = up ? z1 > zb : z1 < zb;
-                                if (!cross || hit == PIC_MAX_HITS) {
-                                    if (cross) c_abs += 1u << 16;            // truncated
-                                    z = cross ? zb : z1;
-                                    if (second) { done = true; break; }
-                                    // the test at mid-step
-                                    second = true;
-                                    tau = half;
-                                    hit = 0;
-                                    if (!bnd || xs < e.P) { sub_ = SUB_EVT; break; }
-                                    continue;
-                                }
-                                const float tb_ = __fdiv_rn(__fsub_rn(zb, z), w);
-                                tau = __fsub_rn(tau, tb_);
+                        const float z1 = fly<DET>(z, w, half), z2 = fly<DET>(z1, w, half);
+                        up = mu > 0.f;
+                        zb = up ? e.hi : e.lo;
+                        const bool bnd = act && (up ? z2 > zb : z2 < zb);
+                        second = !(bnd && (up ? z1 > zb : z1 < zb));     // first event in the second half
+                        sub_ = !bnd ? SUB_EVT : SUB_IF + (second ? 16u : 0u);
+                        const uint4 x = philox_test((uint32_t)slot >> 2, tk, a);
+                        r = philox_rk(make_uint4((uint32_t)slot, ctr_hi, step, sub_), a);
+                        xs = (slot & 2) ? ((slot & 1) ? x.w : x.z) : ((slot & 1) ? x.y : x.x);
+                        const bool scat = xs < e.P;
+                        ev = bnd || (act && scat);
+                        if (!ev) {
+                            z = z2;
+                            sub_ = 0u;
+                        } else {
+                            if (second) z = z1;
+                            if (bnd && second && scat) {
+                                pend = true;
+                                sub_ = 0u;
+                            } else if (bnd) {
+                                tau = __fsub_rn(half, __fdiv_rn(__fsub_rn(zb, z), w));
                                 if (!(tau > 0.f)) tau = 0.f;
                                 z = zb;
-                                if (up ? layer == st.n_layers - 1 : layer == 0) {    // vacuum
-                                    mu = -mu;
-                                    ++hit;
-                                    continue;
-                                }
-                                c_hit += 1u;
-                                if (a.flags & PIC_F_TRANSPARENT) {
-                                    layer += up ? 1 : -1;
-                                    c_hit += 1u << 16;                       // transmitted
-                                    ++hit;
-                                    e = s_ent[(((layer * 2 + sg) << a.kb) + k)];
-                                    continue;
-                                }
-                                sub_ = SUB_IF + (second ? 16u : 0u) + (uint32_t)hit;
-                                break;
                             }
                         }
-                        if (!__any_sync(0xffffffffu, sub_ != 0u)) continue;
-                        const uint4 r = philox_rk(make_uint4((uint32_t)slot, ctr_hi, step, sub_), a);
+                    }
+                    n_event += (uint32_t)__popc(__ballot_sync(0xffffffffu, ev));
+                    bool done = !ev;
+                    uint2 srec = make_uint2(0u, 0u);
+                    // apply the word, fly until the next one is needed or the
+                    // step is done; one Philox call serves every lane
+#pragma unroll 1
+                    for (;;) {
                         if (sub_ == SUB_EVT) {
                             const bool inel = r.y < s_Q[(layer * 2 + sg) * ne + (k - 1)];
                             if (k == 1 && (inel || (a.flags & PIC_F_LOWEST_BIN_ANY))) {
@@ -533,16 +514,57 @@ __global__ void __launch_bounds__(32 * GW_MAX, 1) k_group(const Args a, const Gr
                                 }
                             }
                         } else if (sub_ != 0u) {
-                            const int iface = up ? layer : layer - 1, dir = up ? 0 : 1;
-                            if (r.x < s_T[((iface * 2 + dir) * 2 + sg) * ne + (k - 1)]) {
-                                layer += up ? 1 : -1;
-                                c_hit += 1u << 16;
-                                e = s_ent[(((layer * 2 + sg) << a.kb) + k)];
-                            } else {
-                                mu = -mu;
-                            }
+                            // at the boundary zb
                             ++hit;
+                            if (up ? layer == st.n_layers - 1 : layer == 0) {        // vacuum
+                                mu = -mu;
+                            } else {
+                                const int iface = up ? layer : layer - 1, dir = up ? 0 : 1;
+                                c_hit += 1u;
+                                if ((a.flags & PIC_F_TRANSPARENT) ||
+                                    r.x < s_T[((iface * 2 + dir) * 2 + sg) * ne + (k - 1)]) {
+                                    layer += up ? 1 : -1;
+                                    c_hit += 1u << 16;                       // transmitted
+                                    e = s_ent[(((layer * 2 + sg) << a.kb) + k)];
+                                } else {
+                                    mu = -mu;
+                                }
+                            }
                         }
+                        sub_ = 0u;
+                        if (!done) {
+                            if (pend) {
+                                pend = false;
+                                sub_ = SUB_EVT;
+                            } else {
+#pragma unroll 1
+                                for (;;) {
+                                    const float w = __fmul_rn(e.v, mu);
+                                    const float z1 = fly<DET>(z, w, tau);
+                                    up = mu > 0.f;
+                                    zb = up ? e.hi : e.lo;
+                                    const bool cross = up ? z1 > zb : z1 < zb;
+                                    if (!cross || hit == PIC_MAX_HITS) {
+                                        if (cross) c_abs += 1u << 16;        // truncated
+                                        z = cross ? zb : z1;
+                                        if (second) { done = true; break; }
+                                        // the test at mid-step
+                                        second = true;
+                                        tau = half;
+                                        hit = 0;
+                                        if (xs < e.P) { sub_ = SUB_EVT; break; }
+                                        continue;
+                                    }
+                                    tau = __fsub_rn(tau, __fdiv_rn(__fsub_rn(zb, z), w));
+                                    if (!(tau > 0.f)) tau = 0.f;
+                                    z = zb;
+                                    sub_ = SUB_IF + (second ? 16u : 0u) + (uint32_t)hit;
+                                    break;
+                                }
+                            }
+                        }
+                        if (!__any_sync(0xffffffffu, sub_ != 0u)) break;
+                        r = philox_rk(make_uint4((uint32_t)slot, ctr_hi, step, sub_), a);
                     }
                     // ---- results
                     if (act) {
