@@ -397,7 +397,7 @@ pic_status pic_profile_read(pic_ctx *ctx, pic_kernel_times *out);
  * application whose device memory belongs entirely to its own allocator or
  * pool, or a latency-critical loop that must not allocate.  It runs the same
  * compaction kernel as pic_step, with that kernel's scratch (look-back words
- * for up to 4096 blocks, counters, control block: about 33 KB) held in a
+ * for up to 2^16 tiles, counters, control block: about 0.5 MB) held in a
  * static device array that every GPU which loads the library keeps until
  * the process exits.
  *   z, mu, id, packed (device, read): n slots in the pic_record field layout;

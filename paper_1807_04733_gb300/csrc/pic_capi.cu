@@ -97,7 +97,8 @@ struct pic_ctx {
     DevCounters *d_cnt = nullptr;
     DevCtl *d_ctl = nullptr;
     int64_t total_slots = 0, nh_total = 0, J_total = 0;
-    int n_status = 0;                // look-back words and queue counts allocated
+    int n_status = 0;                // queue counts allocated
+    size_t n_words = 0;              // look-back words allocated
     Args args{};
     LaunchCfg lc{};
     int step = 0;
@@ -709,8 +710,11 @@ pic_status pic_init(pic_ctx **out, const pic_params *p, const pic_stack_desc *st
     const int gmax = std::max({c->lc.grid_fast, c->lc.grid_fast_dep, c->lc.grid_slow,
                                c->lc.grid_slow_dep, c->lc.grid_place, c->lc.grid_place_dep,
                                c->lc.grid_compact, 16 * sms_now});
+    // (the compaction has a look-back word per tile)
+    const size_t n_words = std::max<size_t>(gmax, compact_words(c->total_slots, gmax, n_stacks));
     c->n_status = gmax;
-    if (dalloc(&c->d_status, (size_t)gmax) != cudaSuccess ||
+    c->n_words = n_words;
+    if (dalloc(&c->d_status, n_words) != cudaSuccess ||
         dalloc(&c->d_qcnt, (size_t)gmax) != cudaSuccess ||
         dalloc(&c->d_fspawn, (size_t)gmax) != cudaSuccess) {
         g_init_error = "device allocation of the look-back words";
@@ -790,7 +794,7 @@ pic_status pic_init(pic_ctx **out, const pic_params *p, const pic_stack_desc *st
     if (e == cudaSuccess && !fent.empty()) e = cudaMemcpyAsync(c->d_fent, fent.data(), sizeof(FastEnt) * fent.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && !Tall.empty()) e = cudaMemcpyAsync(c->d_T, Tall.data(), 4 * Tall.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_inj, 0, sizeof(long long) * std::max<size_t>((size_t)n_stacks * 2 * p->n_steps_max, 1), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(unsigned long long) * gmax, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(unsigned long long) * n_words, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_fspawn, 0, sizeof(uint32_t) * gmax, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_bits, 0, 4 * (size_t)(c->total_slots / 32 + 1), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_nh, 0, 4 * (size_t)std::max<int64_t>(c->nh_total, 1), st);
@@ -1394,7 +1398,8 @@ pic_status pic_load(pic_ctx *c, const void *buf, size_t bytes)
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_cnt, cnt.data(), sizeof(DevCounters) * S, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_ctl, &ctl, sizeof(DevCtl), cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(unsigned long long) * c->n_status, c->stream);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(c->d_status, 0, sizeof(unsigned long long) * c->n_words, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_fspawn, 0, sizeof(uint32_t) * c->n_status, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "pic_load copy");
@@ -1734,7 +1739,7 @@ pic_status pic_grad(pic_ctx *c, const float *grad_n, const float *grad_J, double
             for (const LaunchCfg &l : r.lc)
                 r.n_status = std::max({r.n_status, l.grid_fast, l.grid_fast_dep, l.grid_slow,
                                        l.grid_slow_dep, l.grid_place, l.grid_place_dep,
-                                       l.grid_compact});
+                                       (int)compact_words(c->total_slots, l.grid_compact, S)});
         }
         RALLOC(r.status, (size_t)r.n_status);
         RALLOC(r.qcnt, (size_t)r.n_status);

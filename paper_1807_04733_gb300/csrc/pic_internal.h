@@ -27,6 +27,13 @@ constexpr int TPB = 256;            // threads per block of the streaming kernel
 constexpr int VEC = 4;              // particles per thread per tile (128-bit)
 constexpr int TILE = TPB * VEC;     // particles per tile
 constexpr int LEDGER_N = 14;        // fields of pic_ledger
+constexpr int COMPACT_TILE = 16384; // most slots per tile of the compaction
+// look-back words of the compaction of n slots in S stacks by a grid of G blocks
+// (tiles are smaller where the largest would leave blocks without one)
+constexpr long long compact_words(long long n, int G, int S)
+{
+    return (n / COMPACT_TILE > 2ll * G ? n / COMPACT_TILE : 2ll * G) + S;
+}
 
 // ledger field indices (order of pic_ledger)
 enum {
@@ -106,6 +113,7 @@ struct DevCtl {
     unsigned int bar_count;  // grid barrier of the persistent kernel: arrivals,
     unsigned int bar_gen;    //   and its generation
     unsigned int base;       // first step of the graph being replayed (grouped steps)
+    unsigned int ticket;     // next tile of the compaction
 };
 
 struct Args {            // everything a kernel needs, passed by value

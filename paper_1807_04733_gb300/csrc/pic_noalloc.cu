@@ -5,12 +5,12 @@
 // a library allocate or free behind its back), or a latency-critical loop
 // that must not allocate at all.  pic_compact_static lets them run the
 // stable removal of dead slots on particle arrays they own.  The kernel is
-// the library's compaction kernel; its scratch (per-block look-back words,
+// the library's compaction kernel; its scratch (per-tile look-back words,
 // the control block and the counters) lives in the file-scope device array
 // below instead of in a context's allocation.
 //
 // The array is static device memory: every GPU that loads the library holds
-// it (about 33 KB) until the process exits.  All calls on a device share it
+// it (about 0.5 MB) until the process exits.  All calls on a device share it
 // and it keeps the last call's contents, so every call re-initialises the
 // part that must start from a known value; two calls whose kernels overlap
 // on the GPU (different streams, or host threads) race on it.
@@ -26,14 +26,14 @@ using namespace pic;
 
 namespace {
 
-constexpr int kMaxBlocks = 4096;       // look-back words: one per block
+constexpr int kMaxTiles = (int)compact_words(1ll << 30, 0, 1);   // look-back words: one per tile
 constexpr int kMaxDevices = 64;
 
 struct Scratch {
     DevCtl ctl;
     DevCounters cnt;
     DevStack stack;
-    unsigned long long status[kMaxBlocks];
+    unsigned long long status[kMaxTiles];
 };
 
 static __device__ __align__(256) unsigned char g_compact_scratch[sizeof(Scratch)];
@@ -95,7 +95,7 @@ extern "C" pic_status pic_compact_static(const float *z, const float *mu, const 
             e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             if (e != cudaSuccess) return cuda_error(e, "pic_compact_static: SM count");
             d.grid = sms * (2048 / TPB);
-            if (d.grid > kMaxBlocks) d.grid = kMaxBlocks;
+            if (2 * d.grid >= kMaxTiles) d.grid = kMaxTiles / 2 - 1;
             d.ready = true;
         }
         scr = d.addr;

@@ -2127,6 +2127,18 @@ __global__ void __launch_bounds__(TPB) k_inject(const Args a, int half, int depo
 
 // ---------------------------------------------------------------------------
 // k_compact: stable removal of dead slots (k = 0) into the other buffer
+//
+// Tiles of up to COMPACT_TILE slots, taken in order from a ticket.  A block
+// counts its tile's live slots, chains the count by a decoupled look-back over
+// the tiles of the stack (it publishes its count before it waits, so every
+// wait ends), and scatters.  The count reads the packed words (and, interleaved,
+// mu) from memory, the scatter finds them in L2: the tiles in flight are some
+// 60 MB.  (One contiguous chunk per block read them from memory twice; tiles
+// small enough for registers or shared memory were held up by the chain of
+// look-backs, 20 ns a tile.)  A warp takes consecutive slots as rows of 32,
+// lane l the slot l of each row, so that loads and the stores of the live slots
+// are coalesced; a slot's rank is the live slots of the earlier warps, of
+// the earlier rows and of the lower lanes of its row (ballots).
 // ---------------------------------------------------------------------------
 template <int ADJ = 0>
 __device__ __forceinline__ void phase_compact(const Args &a)
@@ -2134,161 +2146,130 @@ __device__ __forceinline__ void phase_compact(const Args &a)
     __shared__ long long s_tpref[PIC_MAX_STACKS + 1];
     __shared__ long long s_nsl[PIC_MAX_STACKS];
     __shared__ int s_w[TPB / 32];
+    __shared__ unsigned int s_tile;
     __shared__ long long s_prefix;
     __shared__ int s_flag;
+    constexpr int CV = 8;                                    // rows at a time
+    constexpr int CS = TPB * CV;                             // smallest tile
     const unsigned int ep = *(volatile unsigned int *)&a.ctl->epoch;
     const int cur = (int)*(volatile unsigned int *)&a.ctl->cur, nxt = cur ^ 1;
-    const int b = blockIdx.x, G = gridDim.x, tid = threadIdx.x;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long S = a.mp_stride;
-    Plan p;
-    make_plan(a, s_tpref, s_nsl, p);
-
-    // Slots are taken in groups of TPB * CV (one tile): warp w takes the
-    // 32 * CV slots [w * 32 CV, (w + 1) * 32 CV) of a group as CV rows of 32, lane l
-    // the slot l of each row, so that loads and the stores of the live slots
-    // are coalesced; a slot's rank is the live slots of the earlier warps
-    // (one block scan of the warps' counts), of the earlier rows and of the
-    // lower lanes of its row (ballots).  A group lies in one stack; lim = the
-    // first slot not in it, or the stack's slot count; nothing at or past lim
-    // is read.
-    constexpr int CV = 4;
-    constexpr long long GT = (long long)TPB * CV / TILE;      // tiles per group
-    const int warp = tid >> 5, lane = tid & 31;
     const unsigned int lt = (1u << lane) - 1u;
-    uint32_t pkv[CV], bal[CV];
-    auto alive_rows = [&](const DevStack &st, long long g0, long long lim) -> int {
-        int n = 0;
-        const long long sl0 = g0 + warp * (32 * CV) + lane;
-        const uint32_t *P = a.pk[cur] + (st.base + sl0) * S;
-        const int left = lim - sl0 > 32 * CV ? 32 * CV : (int)(lim - sl0);   // rows i with i*32 < left
-#pragma unroll
-        for (int i = 0; i < CV; ++i) {
-            pkv[i] = i * 32 < left ? P[i * 32 * S] : 0u;
-            bal[i] = __ballot_sync(0xffffffffu, (pkv[i] & 0xFFu) != 0u);
-            n += __popc(bal[i]);
+    for (int i = tid; i < a.n_stacks; i += TPB) s_nsl[i] = (long long)a.cnt[i].n_slots;
+    cta_sync();
+    // the largest tiles that give every block one
+    long long all = 0;
+    for (int i = 0; i < a.n_stacks; ++i) all += s_nsl[i];
+    const long long per = all / ((long long)gridDim.x * CS);
+    const int K = per < 1 ? 1 : per > COMPACT_TILE / CS ? COMPACT_TILE / CS : (int)per;
+    const int tile = K * CS;
+    if (tid == 0) {
+        long long acc = 0;
+        for (int i = 0; i < a.n_stacks; ++i) {
+            s_tpref[i] = acc;
+            acc += (s_nsl[i] + tile - 1) / tile;
         }
-        return n;                     // the warp's live slots
-    };
-    // exclusive prefix of the warps' counts and the group's total
-    auto warp_scan = [&](int n, int &excl) -> int {
+        s_tpref[a.n_stacks] = acc;
+        s_tile = atomicAdd(&a.ctl->ticket, 1u);
+    }
+    cta_sync();
+    const long long T = s_tpref[a.n_stacks];
+    for (long long t = s_tile; t < T;) {
+        const int s = a.n_stacks == 1 ? 0 : stack_of(s_tpref, a.n_stacks, t);
+        const DevStack &st = a.stacks[s];
+        // the warp's slots: K groups of CV rows; the lane's first one
+        const long long sl0 = (t - s_tpref[s]) * tile + (long long)warp * (32 * CV * K) + lane;
+        const long long left = s_nsl[s] - sl0;               // a row r is read where 32 r < left
+        const uint32_t *P = a.pk[cur] + (st.base + sl0) * S;
+        const float *Zc = a.z[cur] + st.base + sl0;
+        const float *Mc = a.mu[cur] + (st.base + sl0) * S;
+        const uint32_t *Ic = a.id[cur] + st.base + sl0;
+        int n = 0;
+        for (int g = 0; g < K; ++g) {
+            uint32_t pkv[CV];
+#pragma unroll
+            for (int i = 0; i < CV; ++i) {
+                const int r = g * CV + i;
+                pkv[i] = 32 * r < left ? P[32 * r * S] : 0u;
+            }
+#pragma unroll
+            for (int i = 0; i < CV; ++i) n += __popc(__ballot_sync(0xffffffffu, (pkv[i] & 0xFFu) != 0u));
+        }
         if (lane == 0) s_w[warp] = n;
         cta_sync();
-        int pre = 0, tot = 0;
+        int excl = 0, tot = 0;
 #pragma unroll
         for (int w = 0; w < TPB / 32; ++w) {
             const int v = s_w[w];
-            pre += w < warp ? v : 0;
+            excl += w < warp ? v : 0;
             tot += v;
         }
-        cta_sync();
-        excl = pre;
-        return tot;
-    };
-    // the groups of stack s inside this block's chunk: [ta, tb) tiles
-    auto seg_tiles = [&](int s, long long &ta, long long &tb) {
-        ta = p.t0 > s_tpref[s] ? p.t0 : s_tpref[s];
-        tb = p.t1 < s_tpref[s + 1] ? p.t1 : s_tpref[s + 1];
-    };
-
-    if (p.t0 < p.t1) {
-        const int s_first = stack_of(s_tpref, a.n_stacks, p.t0);
-        const int s_last = stack_of(s_tpref, a.n_stacks, p.t1 - 1);
-        const bool first_inside = p.t0 > s_tpref[s_first];
-        // phase 1: count the first segment (if it needs the look-back) and the
-        // last segment (its count is what later blocks need)
-        long long c_first = 0, c_last = 0;
-        for (int s = s_first; s <= s_last; ++s) {
-            const bool need = (s == s_first && first_inside) || s == s_last;
-            if (!need) continue;
-            const DevStack &st = a.stacks[s];
-            long long ta, tb;
-            seg_tiles(s, ta, tb);
-            for (long long t = ta; t < tb; t += GT) {
-                const long long g0 = (t - s_tpref[s]) * TILE;
-                const long long ge = ((t + GT < tb ? t + GT : tb) - s_tpref[s]) * TILE;
-                int excl;
-                const int tot = warp_scan(alive_rows(st, g0, ge < s_nsl[s] ? ge : s_nsl[s]), excl);
-                if (s == s_first) c_first += tot;
-                if (s == s_last) c_last += tot;
-            }
-        }
-        long long pre_first = 0;
         if (tid < 32) {
-            // the look-back takes the whole warp
-            if (s_last == s_first && first_inside) {
-                if (tid == 0) publish(&a.status[b], ep, FLAG_A, c_last);
-                const long long pre = look_back(a, ep, p.T, s_tpref[s_first], b, G);
-                if (tid == 0) {
-                    s_prefix = pre;
-                    publish(&a.status[b], ep, FLAG_P, pre + c_last);
-                }
-            } else {
-                if (tid == 0) publish(&a.status[b], ep, FLAG_P, c_last);
-                const long long pre = first_inside ? look_back(a, ep, p.T, s_tpref[s_first], b, G) : 0;
-                if (tid == 0) s_prefix = pre;
+            // (a status word says everything itself: no fence)
+            const unsigned long long tag = (unsigned long long)ep << 32;
+            volatile unsigned long long *word = &a.status[t];
+            long long pre = 0;
+            if (t > s_tpref[s]) {
+                if (tid == 0) *word = tag | (FLAG_A << 30) | (unsigned long long)tot;
+                pre = look_back_warp(a, ep, s_tpref[s], (int)t, [](int j) { return (long long)j; });
+            }
+            if (tid == 0) {
+                *word = tag | (FLAG_P << 30) | (unsigned long long)(pre + tot);
+                s_prefix = pre;
+                if (t + 1 == s_tpref[s + 1]) a.cnt[s].alive_total = (unsigned long long)(pre + tot);
             }
         }
         cta_sync();
-        pre_first = s_prefix;
-        (void)c_first;
-        // phase 2: scatter live slots, stable, into the other buffer
-        for (int s = s_first; s <= s_last; ++s) {
-            const DevStack &st = a.stacks[s];
-            long long ta, tb;
-            seg_tiles(s, ta, tb);
-            if (ta >= tb) continue;
-            long long run = (s == s_first) ? pre_first : 0;
-            for (long long t = ta; t < tb; t += GT) {
-                const long long g0 = (t - s_tpref[s]) * TILE;
-                const long long ge = ((t + GT < tb ? t + GT : tb) - s_tpref[s]) * TILE;
-                const long long lim = ge < s_nsl[s] ? ge : s_nsl[s];
-                const long long sl0 = g0 + warp * (32 * CV) + lane;  // this lane's first slot
-                const int left = lim - sl0 > 32 * CV ? 32 * CV : (int)(lim - sl0);
-                const float *Zc = a.z[cur] + st.base + sl0;
-                const float *Mc = a.mu[cur] + (st.base + sl0) * S;
-                const uint32_t *Ic = a.id[cur] + st.base + sl0;
-                float zv[CV], muv[CV];
-                uint32_t idv[CV];
+        long long d = st.base + s_prefix + excl;
+        for (int g = 0; g < K; ++g) {
+            float zv[CV], muv[CV];
+            uint32_t idv[CV], pkv[CV];
 #pragma unroll
-                for (int i = 0; i < CV; ++i) {
-                    const bool in = i * 32 < left;
-                    zv[i] = in ? Zc[i * 32] : 0.f;
-                    muv[i] = in ? Mc[i * 32 * S] : 0.f;
-                    idv[i] = in ? Ic[i * 32] : 0u;
+            for (int i = 0; i < CV; ++i) {
+                const int r = g * CV + i;
+                const bool in = 32 * r < left;
+                if (S == 2) {
+                    const uint2 mp = in ? *reinterpret_cast<const uint2 *>(Mc + 64 * r) : make_uint2(0u, 0u);
+                    muv[i] = __uint_as_float(mp.x);
+                    pkv[i] = mp.y;
+                } else {
+                    muv[i] = in ? Mc[32 * r] : 0.f;
+                    pkv[i] = in ? P[32 * r] : 0u;
                 }
-                int excl;
-                const int tot = warp_scan(alive_rows(st, g0, lim), excl);
-                long long d = st.base + run + excl;
-#pragma unroll
-                for (int i = 0; i < CV; ++i) {
-                    const long long src = st.base + sl0 + i * 32;
-                    if ((bal[i] >> lane) & 1u) {
-                        const long long o = d + __popc(bal[i] & lt);
-                        a.z[nxt][o] = zv[i];
-                        if (S == 2) {
-                            *reinterpret_cast<uint2 *>(a.mu[nxt] + 2 * o) =
-                                make_uint2(__float_as_uint(muv[i]), pkv[i]);
-                        } else {
-                            a.mu[nxt][o] = muv[i];
-                            a.pk[nxt][o] = pkv[i];
-                        }
-                        a.id[nxt][o] = idv[i];
-                        if (!ADJ && a.w[0]) a.w[nxt][o] = a.w[cur][src];
-                        if (ADJ) a.acc[nxt][o] = a.acc[cur][src];
-                    } else if (ADJ == 1 && i * 32 < left) {
-                        // pass 1: a removed carrier's own reward is final
-                        const unsigned long long id = (unsigned long long)idv[i] |
-                                                      ((unsigned long long)(pkv[i] >> 21) << 32);
-                        if (id < (unsigned long long)st.n_ids) a.tot[st.id_off + (long long)id] = a.acc[cur][src];
-                        else atomicCAS(&a.ctl->status, 0u, (unsigned int)PIC_ERR_STATE);
-                    }
-                    d += __popc(bal[i]);
-                }
-                run += tot;
+                zv[i] = in ? Zc[32 * r] : 0.f;
+                idv[i] = in ? Ic[32 * r] : 0u;
             }
-            if (s_tpref[s + 1] <= p.t1 && tid == 0)
-                a.cnt[s].alive_total = (unsigned long long)run;
+#pragma unroll
+            for (int i = 0; i < CV; ++i) {
+                const unsigned int bal = __ballot_sync(0xffffffffu, (pkv[i] & 0xFFu) != 0u);
+                const long long src = st.base + sl0 + 32 * (g * CV + i);
+                if ((bal >> lane) & 1u) {
+                    const long long o = d + __popc(bal & lt);
+                    a.z[nxt][o] = zv[i];
+                    if (S == 2) {
+                        *reinterpret_cast<uint2 *>(a.mu[nxt] + 2 * o) = make_uint2(__float_as_uint(muv[i]), pkv[i]);
+                    } else {
+                        a.mu[nxt][o] = muv[i];
+                        a.pk[nxt][o] = pkv[i];
+                    }
+                    a.id[nxt][o] = idv[i];
+                    if (!ADJ && a.w[0]) a.w[nxt][o] = a.w[cur][src];
+                    if (ADJ) a.acc[nxt][o] = a.acc[cur][src];
+                } else if (ADJ == 1 && 32 * (g * CV + i) < left) {
+                    // pass 1: a removed carrier's own reward is final
+                    const unsigned long long id = (unsigned long long)idv[i] |
+                                                  ((unsigned long long)(pkv[i] >> 21) << 32);
+                    if (id < (unsigned long long)st.n_ids) a.tot[st.id_off + (long long)id] = a.acc[cur][src];
+                    else atomicCAS(&a.ctl->status, 0u, (unsigned int)PIC_ERR_STATE);
+                }
+                d += __popc(bal);
+            }
         }
+        // (a ticket taken earlier would hold up the tiles behind it)
+        if (tid == 0) s_tile = atomicAdd(&a.ctl->ticket, 1u);
+        cta_sync();
+        t = s_tile;
     }
 
     if (last_block(a, &s_flag)) {
@@ -2300,13 +2281,14 @@ __device__ __forceinline__ void phase_compact(const Args &a)
         if (tid == 0) {
             a.ctl->cur = (unsigned int)nxt;
             a.ctl->done = 0u;
+            a.ctl->ticket = 0u;
             a.ctl->epoch = ep + 1u;
         }
     }
 }
 
 template <int ADJ = 0>
-__global__ void __launch_bounds__(TPB) k_compact(const Args a)
+__global__ void __launch_bounds__(TPB, 4) k_compact(const Args a)
 {
     phase_compact<ADJ>(a);
 }
