@@ -119,6 +119,7 @@ struct pic_ctx {
     int64_t period_launches[2] = {0, 0};
     int period = 0;
     bool dev_step_valid = false;     // d_ctl->step == step
+    int src_end = 0;                 // first step after which no source carrier comes
     // the persistent kernel (use_graph 2): its configuration and the graph of
     // one launch covering a period
     PersistCfg pcfg;
@@ -134,6 +135,7 @@ struct pic_ctx {
     GroupRes *d_gres = nullptr;
     unsigned int *d_gbar = nullptr;
     int4 *d_gblk = nullptr;
+    GroupArgs ga_run{};              // the same for the persistent form's grid
     // kernel timing (pic_profile)
     bool profiling = false;
     std::vector<cudaEvent_t> ev_pool;
@@ -427,6 +429,19 @@ cudaError_t timed(pic_ctx *c, int kind, F fn)
         c->ev_marks.push_back({kind, i});
         c->ev_used += 2;
     }
+    return e;
+}
+
+// First step after which no stack's source creates a carrier.
+int source_end(const pic_ctx *c)
+{
+    int e = 0;
+    for (const HostStack &h : c->hs)
+        for (int64_t i = (int64_t)h.inj.size() - 1; i >= 2 * (int64_t)e; --i)
+            if (h.inj[(size_t)i] > 0) {
+                e = (int)(i / 2) + 1;
+                break;
+            }
     return e;
 }
 
@@ -732,29 +747,35 @@ pic_status pic_init(pic_ctx **out, const pic_params *p, const pic_stack_desc *st
     std::vector<int4> blk;
     if (e == cudaSuccess && c->gc.ok) {
         GroupArgs &g = c->ga;
-        const int gt = c->gc.grid_tail;
+        const int gt = c->gc.grid_tail, gr = c->gc.grid, gmx = std::max(gt, gr);
         g.cnt_n = c->total_slots / GROUP_SUB_MIN + 1;
         e = dalloc(&c->d_gcnt, (size_t)GROUP_OPEN * g.cnt_n);
         if (e == cudaSuccess) e = dalloc(&c->d_gabs, (size_t)n_stacks * GROUP_MAX);
-        if (e == cudaSuccess) e = dalloc(&c->d_gsum, (size_t)2 * GROUP_OPEN * gt);
+        if (e == cudaSuccess) e = dalloc(&c->d_gsum, (size_t)2 * GROUP_OPEN * gmx);
         if (e == cudaSuccess) e = dalloc(&c->d_gres, n_stacks);
-        if (e == cudaSuccess) e = dalloc(&c->d_gbar, (size_t)2 * n_stacks);
-        if (e == cudaSuccess) e = dalloc(&c->d_gblk, gt);
+        if (e == cudaSuccess) e = dalloc(&c->d_gbar, (size_t)32 * n_stacks);
+        if (e == cudaSuccess) e = dalloc(&c->d_gblk, gt + gr);
         // every stack one block, the others by capacity (the rest to the largest)
-        std::vector<int> nb(n_stacks, 1);
-        int left = gt - n_stacks, big = 0;
-        const int spare = left;
-        for (int s = 0; s < n_stacks; ++s) {
-            const int add = (int)((double)spare * (double)c->hs[s].cap_round / (double)std::max<int64_t>(c->total_slots, 1));
-            nb[s] += std::min(add, left);
-            left -= std::min(add, left);
-            if (c->hs[s].cap_round > c->hs[big].cap_round) big = s;
-        }
-        nb[big] += left;
-        for (int s = 0; s < n_stacks; ++s) {
-            const int first = (int)blk.size();
-            for (int i = 0; i < nb[s]; ++i) blk.push_back(make_int4(s, i, nb[s], first));
-        }
+        auto share = [&](int total) {
+            std::vector<int> nb(n_stacks, 1);
+            int left = total - n_stacks, big = 0;
+            const int spare = left;
+            for (int s = 0; s < n_stacks; ++s) {
+                const int add = std::min(left, (int)((double)spare * (double)c->hs[s].cap_round /
+                                                     (double)std::max<int64_t>(c->total_slots, 1)));
+                nb[s] += add;
+                left -= add;
+                if (c->hs[s].cap_round > c->hs[big].cap_round) big = s;
+            }
+            nb[big] += left;
+            int first = 0;
+            for (int s = 0; s < n_stacks; ++s) {
+                for (int i = 0; i < nb[s]; ++i) blk.push_back(make_int4(s, i, nb[s], first));
+                first += nb[s];
+            }
+        };
+        share(gt);
+        if (c->gc.run) share(gr);
         // the lists of the four steps: one 8-byte record per slot and step, in
         // the buffers of the single steps' staged and queued records
         g.list[0] = reinterpret_cast<uint2 *>(c->d_stage);
@@ -763,13 +784,16 @@ pic_status pic_init(pic_ctx **out, const pic_params *p, const pic_stack_desc *st
         g.cnt = c->d_gcnt;
         g.abs = c->d_gabs;
         g.bsum = c->d_gsum;
-        g.tsum = c->d_gsum + (size_t)GROUP_OPEN * gt;
+        g.tsum = c->d_gsum + (size_t)GROUP_OPEN * gmx;
         g.res = c->d_gres;
         g.bar = c->d_gbar;
         g.blk = c->d_gblk;
         g.sub = 128 * c->gc.quads;
         g.nd = c->gc.nd;
         g.nj = c->gc.nj;
+        g.m = c->gc.m;
+        c->ga_run = g;
+        c->ga_run.blk = c->d_gblk + gt;
     }
     if (e != cudaSuccess) {
         g_init_error = std::string("grouped steps: ") + cudaGetErrorString(e);
@@ -784,7 +808,7 @@ pic_status pic_init(pic_ctx **out, const pic_params *p, const pic_stack_desc *st
     ctl.epoch = 1u;
     if (c->gc.ok) {
         e = cudaMemsetAsync(c->d_gabs, 0, sizeof(uint32_t) * (size_t)n_stacks * GROUP_MAX, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->d_gbar, 0, sizeof(unsigned int) * 2 * (size_t)n_stacks, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->d_gbar, 0, sizeof(unsigned int) * 32 * (size_t)n_stacks, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_gblk, blk.data(), sizeof(int4) * blk.size(), cudaMemcpyHostToDevice, st);
     }
     std::vector<DevCounters> cnt(n_stacks);
@@ -890,6 +914,10 @@ pic_status pic_excite(pic_ctx *c, int stack, const pic_pulse *u)
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "pic_excite upload");
     }
+    c->src_end = source_end(c);
+    // (a captured launch carries it)
+    if (c->persist_graph) cudaGraphExecDestroy(c->persist_graph);
+    c->persist_graph = nullptr;
     return PIC_OK;
 }
 
@@ -1018,6 +1046,21 @@ cudaError_t enqueue_range(pic_ctx *c, const Args &a0, int s, int e, const unsign
     return r;
 }
 
+// Whether single launches give way to the persistent form: few carriers, where
+// the gaps between the launches of a group count (a run of 500 steps from 1e5
+// carriers 9.1 -> 8.4 ms, one of 600 steps from 1.2e6 carriers 28.8 -> 28.4;
+// with more, its one block per SM is too few for the new carriers).
+bool run_plain(const pic_ctx *c) { return c->gc.run && !c->profiling && c->total_slots <= (8ll << 20); }
+
+// n_steps whole steps in one persistent launch of grouped steps
+cudaError_t enqueue_run(pic_ctx *c, int n_steps, cudaStream_t st)
+{
+    Args a = c->args;
+    a.step_dev = &c->d_ctl->step;
+    a.bump_step = 0;
+    return launch_run(a, c->ga_run, c->gc, (c->p.flags & PIC_F_DETERMINISTIC) != 0, n_steps, c->src_end, st);
+}
+
 // Capture one period of steps (starting at a step that is a multiple of the
 // period) into a graph; with_source: the source kernels of every half step.
 cudaError_t capture_period(pic_ctx *c, int which)
@@ -1124,7 +1167,8 @@ pic_status pic_step(pic_ctx *c, int n_steps)
         if (persist && c->period > 0 && s % c->period == 0 && left >= c->period) {
             // one cooperative launch runs the whole period (captured in a
             // graph once; the kernel reads and advances the device step)
-            if (!c->pcfg.ok) {
+            const bool run = grouped(c) && c->gc.run;
+            if (!run && !c->pcfg.ok) {
                 e = configure_persistent(c->args, (c->p.flags & PIC_F_DETERMINISTIC) != 0, &c->pcfg);
                 if (e != cudaSuccess) return cuda_fail(c, e, "pic_step persistent configuration");
                 if (c->pcfg.grid > c->n_status)
@@ -1138,7 +1182,8 @@ pic_status pic_step(pic_ctx *c, int n_steps)
                 cudaGraph_t g = nullptr;
                 if (e == cudaSuccess) e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
                 if (e == cudaSuccess) {
-                    cudaError_t e1 = launch_persistent(a, c->pcfg, det, c->period, c->cap_stream);
+                    cudaError_t e1 = run ? enqueue_run(c, c->period, c->cap_stream)
+                                         : launch_persistent(a, c->pcfg, det, c->period, c->cap_stream);
                     cudaError_t e2 = cudaStreamEndCapture(c->cap_stream, &g);
                     if (e1 == cudaSuccess && e2 == cudaSuccess)
                         e1 = cudaGraphInstantiate(&c->persist_graph, g, 0);
@@ -1157,6 +1202,7 @@ pic_status pic_step(pic_ctx *c, int n_steps)
             }
             if (e == cudaSuccess)
                 e = c->persist_graph ? cudaGraphLaunch(c->persist_graph, c->stream)
+                    : run            ? enqueue_run(c, c->period, c->stream)
                                      : launch_persistent(a, c->pcfg, det, c->period, c->stream);
             if (e != cudaSuccess) return cuda_fail(c, e, "pic_step persistent launch");
             c->dev_step_valid = true;
@@ -1184,12 +1230,18 @@ pic_status pic_step(pic_ctx *c, int n_steps)
             continue;
         }
         if (grouped(c)) {
-            const int s1 = std::min(range_end(c, s), s + left);
+            const bool run = run_plain(c) && left > c->gc.m;
+            const int s1 = run ? s + left : std::min(range_end(c, s), s + left);
             if (!c->dev_step_valid) {
                 e = launch_set_step(c->d_ctl, (unsigned int)s, c->stream);
                 c->launches += 1;
             }
-            if (e == cudaSuccess) e = enqueue_range(c, c->args, s, s1, nullptr, false, c->stream, c->launches);
+            if (e == cudaSuccess && run) {
+                e = timed(c, 1, [&] { return enqueue_run(c, left, c->stream); });
+                c->launches += 1;
+            } else if (e == cudaSuccess) {
+                e = enqueue_range(c, c->args, s, s1, nullptr, false, c->stream, c->launches);
+            }
             if (e != cudaSuccess) return cuda_fail(c, e, "pic_step launch");
             c->dev_step_valid = true;
             c->step = s1;

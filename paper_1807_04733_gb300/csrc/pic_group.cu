@@ -114,22 +114,20 @@ struct Span {
 };
 
 template <bool DEP>
-__device__ __forceinline__ Span group_span(const Args &a, const GroupArgs &g)
+__device__ __forceinline__ Span group_span(const Args &a, uint32_t s0, int span, int m, bool no_src)
 {
     Span sp{};
-    const uint32_t base = g.base ? __ldcg(g.base) : 0u;
-    sp.s0 = base + (uint32_t)g.off;
-    if (__ldcg(&a.ctl->step) != sp.s0) return sp;
-    bool closed = g.no_src != 0;
+    sp.s0 = s0;
+    if (__ldcg(&a.ctl->step) != s0) return sp;
+    bool open = !no_src;
     if (!(a.flags & PIC_F_NO_SECONDARIES))
-        for (int s = threadIdx.x; s < a.n_stacks; s += (int)blockDim.x) {
+        for (int s = threadIdx.x; s < a.n_stacks; s += TPB) {
             const long long n = (long long)__ldcg(&a.cnt[s].n_slots);
-            if (n > 0 && n < a.stacks[s].cap) closed = false;
+            if (n > 0 && n < a.stacks[s].cap) open = true;
         }
-    sp.closed = __syncthreads_and(closed) != 0;
-    const int span = g.end - g.off;
+    sp.closed = !cta_sync_or(open);
     // densities inside the group: as many steps as windows are held
-    sp.len = sp.closed && !DEP ? span : (g.m < span ? g.m : span);
+    sp.len = sp.closed && !DEP ? span : (m < span ? m : span);
     return sp;
 }
 
@@ -200,7 +198,7 @@ __host__ __device__ inline GroupSmem group_smem(const Args &a, bool dep, int qua
 // threshold 0.
 // ---------------------------------------------------------------------------
 template <bool DET, bool DEP, int Q>
-__global__ void __launch_bounds__(32 * GW_MAX, 1) k_group(const Args a, const GroupArgs g)
+__device__ __forceinline__ void phase_group(const Args &a, const GroupArgs &g, const Span sp)
 {
     constexpr int S = 128 * Q;               // slots of a sub-tile
     constexpr int RQ = Q + 1;                // padded row of a lane, vectors
@@ -210,8 +208,6 @@ __global__ void __launch_bounds__(32 * GW_MAX, 1) k_group(const Args a, const Gr
     __shared__ unsigned long long s_led[9];
     __shared__ unsigned int s_next;
 
-    const Span sp = group_span<DEP>(a, g);
-    if (sp.len == 0) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NT = (int)blockDim.x;
     const GroupSmem o = group_smem(a, DEP, Q, 0, g.nd, g.nj);
     FastEnt *s_ent = reinterpret_cast<FastEnt *>(smem + o.ent);
@@ -685,6 +681,28 @@ __global__ void __launch_bounds__(32 * GW_MAX, 1) k_group(const Args a, const Gr
     }
 }
 
+// The span is decided by the block's first TPB threads (the width of k_tail's
+// blocks, which decide the same) and handed to the others.
+template <bool DEP>
+__device__ __forceinline__ Span block_span(const Args &a, uint32_t s0, int span, int m, bool no_src)
+{
+    __shared__ Span s_sp;
+    if (threadIdx.x < TPB) {
+        const Span sp = group_span<DEP>(a, s0, span, m, no_src);
+        if (threadIdx.x == 0) s_sp = sp;
+    }
+    __syncthreads();
+    return s_sp;
+}
+
+template <bool DET, bool DEP, int Q>
+__global__ void __launch_bounds__(32 * GW_MAX, 1) k_group(const Args a, const GroupArgs g)
+{
+    const uint32_t s0 = (g.base ? __ldcg(g.base) : 0u) + (uint32_t)g.off;
+    const Span sp = block_span<DEP>(a, s0, g.end - g.off, g.m, g.no_src != 0);
+    if (sp.len != 0) phase_group<DET, DEP, Q>(a, g, sp);
+}
+
 // ---------------------------------------------------------------------------
 // k_tail: the carriers created in the steps of an open group.  Every stack has
 // blocks of its own (in proportion to its capacity) with a barrier among them;
@@ -710,34 +728,28 @@ __device__ __forceinline__ void agg_sum(unsigned long long *p, uint32_t v)
     if ((int)(threadIdx.x & 31) == __ffs(m) - 1) atomicAdd(p, (unsigned long long)t);
 }
 
-// barrier of the stack's nb blocks (all resident: a cooperative launch), as
-// grid_sync: sense by generation, the wait bounded in polls
-__device__ __forceinline__ void stack_sync(const Args &a, unsigned int *bar, unsigned int nb)
+// Barrier of the stack's nb blocks (all resident: a cooperative launch): one
+// counter that only grows, `target` the arrivals that end this barrier.  One
+// trip to memory to arrive, then polls; bounded in polls.
+__device__ __forceinline__ void stack_sync(const Args &a, unsigned int *bar, unsigned int target)
 {
-    __syncthreads();
+    cta_sync();
     if (threadIdx.x == 0) {
-        volatile unsigned int *gen = bar + 1;
-        const unsigned int g0 = *gen;
-        __threadfence();
-        if (atomicAdd(bar, 1u) == nb - 1) {
-            *(volatile unsigned int *)bar = 0u;
-            __threadfence();
-            atomicAdd(bar + 1, 1u);
-        } else {
-            unsigned int it = 0;
-            while (*gen == g0) {
-                if (++it > a.spin_limit) {
-                    atomicCAS(&a.ctl->status, 0u, (unsigned int)PIC_ERR_TIMEOUT);
-                    a.ctl->timeout_where = 7u;
-                    break;
-                }
-                if (*(volatile unsigned int *)&a.ctl->status == (unsigned int)PIC_ERR_TIMEOUT) break;
-                if (it > 256) __nanosleep(128);
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        unsigned int it = 0, v;
+        for (;;) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            if ((int)(v - target) >= 0) break;
+            if (++it > a.spin_limit) {
+                atomicCAS(&a.ctl->status, 0u, (unsigned int)PIC_ERR_TIMEOUT);
+                a.ctl->timeout_where = 7u;
+                break;
             }
+            if ((it & 63u) == 0 && *(volatile unsigned int *)&a.ctl->status == (unsigned int)PIC_ERR_TIMEOUT) break;
+            if (it > 1024) __nanosleep(128);
         }
-        __threadfence();
     }
-    __syncthreads();
+    cta_sync();
 }
 
 struct TailStack {                   // what a tail block keeps of its stack
@@ -823,7 +835,7 @@ __device__ __forceinline__ void tail_source(const Args &a, const TailStack &x, u
 }
 
 template <bool DET>
-__global__ void __launch_bounds__(TPB, 2) k_tail(const Args a, const GroupArgs g)
+__device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, const Span sp, bool no_src)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     TabEnt *s_ent = reinterpret_cast<TabEnt *>(smem);
@@ -837,11 +849,10 @@ __global__ void __launch_bounds__(TPB, 2) k_tail(const Args a, const GroupArgs g
     __shared__ int s_w[TPB / 32], s_flag;
     __shared__ unsigned long long s_r8[(TPB / 32) * 10];
 
-    const Span sp = g.nd > 0 ? group_span<true>(a, g) : group_span<false>(a, g);
-    if (sp.len == 0) return;
     const int tid = threadIdx.x, lane = tid & 31;
     const int4 bl = g.blk[blockIdx.x];
     const int s = bl.x, ib = bl.y, nbk = bl.z, b0 = bl.w;
+    unsigned int *bar = g.bar + 32 * s, bar_t = 0;       // the last block of the launch resets it
     unsigned long long psum = 0, adds = 0;       // advanced carriers and created ones, without removals
     const unsigned long long live0 = __ldcg(&a.cnt[s].live);
     const long long n0 = (long long)__ldcg(&a.cnt[s].n_slots);
@@ -885,7 +896,7 @@ __global__ void __launch_bounds__(TPB, 2) k_tail(const Args a, const GroupArgs g
         }
         cta_sync();
         if (tid < sp.len) g.bsum[(long long)(b0 + ib) * GROUP_OPEN + tid] = s_tot[tid];
-        stack_sync(a, g.bar + 2 * s, (unsigned int)nbk);
+        stack_sync(a, bar, bar_t += (unsigned int)nbk);
         if (tid < GROUP_OPEN) s_tot[tid] = 0u;
         cta_sync();
         for (int i = tid; i < nbk * sp.len; i += TPB) {
@@ -905,7 +916,7 @@ __global__ void __launch_bounds__(TPB, 2) k_tail(const Args a, const GroupArgs g
             const bool dep = dep_in && (step + 1) % me == 0;
             uint2 *list = list_of(g, j) + st.base;
             // ---- the source's first half: slots [nsl, nsl + i0)
-            const long long in0 = g.no_src ? 0 : a.inj[st.inj_off + 2 * (long long)step];
+            const long long in0 = no_src ? 0 : a.inj[st.inj_off + 2 * (long long)step];
             const long long r0 = st.cap - nsl;
             const long long i0 = in0 < r0 ? in0 : (r0 > 0 ? r0 : 0);
             psum += live0 + adds + (unsigned long long)i0;
@@ -1000,7 +1011,7 @@ __global__ void __launch_bounds__(TPB, 2) k_tail(const Args a, const GroupArgs g
                 if (lane == 0 && mine) atomicAdd(&s_tt[0], mine);
                 cta_sync();
                 if (tid == 0) g.tsum[(long long)(b0 + ib) * GROUP_OPEN + j] = s_tt[0];
-                stack_sync(a, g.bar + 2 * s, (unsigned int)nbk);
+                stack_sync(a, bar, bar_t += (unsigned int)nbk);
                 if (tid == 0) s_tt[0] = 0u;
                 cta_sync();
                 for (int b = tid; b < nbk; b += TPB) {
@@ -1112,7 +1123,7 @@ __global__ void __launch_bounds__(TPB, 2) k_tail(const Args a, const GroupArgs g
             nsl += kept;
             nid += (unsigned long long)kept;
             // ---- the source's second half: slots [nsl, nsl + i1), not moved
-            const long long in1 = g.no_src ? 0 : a.inj[st.inj_off + 2 * (long long)step + 1];
+            const long long in1 = no_src ? 0 : a.inj[st.inj_off + 2 * (long long)step + 1];
             const long long r1 = st.cap - nsl;
             const long long i1 = in1 < r1 ? in1 : (r1 > 0 ? r1 : 0);
             for (long long xi = (long long)ib * TPB + tid; xi < i1; xi += (long long)nbk * TPB)
@@ -1128,7 +1139,7 @@ __global__ void __launch_bounds__(TPB, 2) k_tail(const Args a, const GroupArgs g
             nid += (unsigned long long)i1;
             adds += (unsigned long long)(i0 + kept + i1);
             // the carriers written here are read by other blocks in the next step
-            if (j + 1 < sp.len && nsl > n0) stack_sync(a, g.bar + 2 * s, (unsigned int)nbk);
+            if (j + 1 < sp.len && nsl > n0) stack_sync(a, bar, bar_t += (unsigned int)nbk);
         }
         // ---- the block's counts
         const uint32_t vals[10] = {ty.absorbed, ty.bath, ty.hits, ty.trans, ty.trunc, ty.spawn_drop,
@@ -1161,6 +1172,7 @@ __global__ void __launch_bounds__(TPB, 2) k_tail(const Args a, const GroupArgs g
                 gone += c;
                 gone_steps += c * (unsigned long long)(sp.len - 1 - j);
             }
+            g.bar[32 * q] = 0u;
             DevCounters &c = a.cnt[q];
             c.n_slots = r.n_slots;
             c.next_id = r.next_id;
@@ -1174,6 +1186,15 @@ __global__ void __launch_bounds__(TPB, 2) k_tail(const Args a, const GroupArgs g
     }
 }
 
+template <bool DET>
+__global__ void __launch_bounds__(TPB, 2) k_tail(const Args a, const GroupArgs g)
+{
+    const uint32_t s0 = (g.base ? __ldcg(g.base) : 0u) + (uint32_t)g.off;
+    const Span sp = g.nd > 0 ? group_span<true>(a, s0, g.end - g.off, g.m, g.no_src != 0)
+                             : group_span<false>(a, s0, g.end - g.off, g.m, g.no_src != 0);
+    if (sp.len != 0) phase_tail<DET>(a, g, sp, g.no_src != 0);
+}
+
 // ---------------------------------------------------------------------------
 // k_dens: the densities, generation and velocity sums of the window that the
 // step before ended, from the state: 12 bytes read per slot and two or three
@@ -1181,8 +1202,9 @@ __global__ void __launch_bounds__(TPB, 2) k_tail(const Args a, const GroupArgs g
 // ---------------------------------------------------------------------------
 constexpr int DENS_T = 512;
 
-__global__ void __launch_bounds__(DENS_T) k_dens(const Args a)
+__device__ __forceinline__ void phase_dens(const Args &a)
 {
+    const int NT = (int)blockDim.x;
     extern __shared__ __align__(128) unsigned char smem[];
     uint32_t *s_n = reinterpret_cast<uint32_t *>(smem);
     uint32_t *s_gs = s_n + a.nbin_max;
@@ -1196,7 +1218,7 @@ __global__ void __launch_bounds__(DENS_T) k_dens(const Args a)
     const int tid = threadIdx.x, ne = a.n_e;
     const int cur = (int)__ldcg(&a.ctl->cur);
     const int t = (int)(__ldcg(&a.ctl->step) / (uint32_t)a.moment_every) - 1;
-    for (int s = tid; s < a.n_stacks; s += DENS_T) s_nsl[s] = (long long)a.cnt[s].n_slots;
+    for (int s = tid; s < a.n_stacks; s += NT) s_nsl[s] = (long long)a.cnt[s].n_slots;
     __syncthreads();
     if (tid == 0) {
         long long acc = 0;
@@ -1218,11 +1240,11 @@ __global__ void __launch_bounds__(DENS_T) k_dens(const Args a)
         const DevStack &st = a.stacks[s];
         const int nc = st.n_cells, nb = 2 * ne * nc;
         __syncthreads();
-        for (int i = tid; i < nb; i += DENS_T) s_n[i] = 0u;
-        for (int i = tid; i < nc; i += DENS_T) s_gs[i] = 0u;
+        for (int i = tid; i < nb; i += NT) s_n[i] = 0u;
+        for (int i = tid; i < nc; i += NT) s_gs[i] = 0u;
         if (vmom) {
-            for (int i = tid; i < 2 * nc; i += DENS_T) s_v[i] = 0ull;
-            for (int i = tid; i < st.ftab_n; i += DENS_T) s_ent[i] = a.fent[st.fent_off + i];
+            for (int i = tid; i < 2 * nc; i += NT) s_v[i] = 0ull;
+            for (int i = tid; i < st.ftab_n; i += NT) s_ent[i] = a.fent[st.fent_off + i];
         }
         __syncthreads();
         const float *Z = a.z[cur] + st.base;
@@ -1231,7 +1253,7 @@ __global__ void __launch_bounds__(DENS_T) k_dens(const Args a)
         long long i1 = (tb - s_tpref[s]) * TILE;
         if (i1 > s_nsl[s]) i1 = s_nsl[s];
 #pragma unroll 2
-        for (long long i = i0 + 4 * tid; i < i1; i += 4 * DENS_T) {
+        for (long long i = i0 + 4 * tid; i < i1; i += 4 * NT) {
             const float4 z4 = *reinterpret_cast<const float4 *>(Z + i);
             const uint4 *mp = reinterpret_cast<const uint4 *>(MU + 2 * i);
             const uint4 m0 = mp[0], m1 = mp[1];
@@ -1254,15 +1276,62 @@ __global__ void __launch_bounds__(DENS_T) k_dens(const Args a)
         __syncthreads();
         uint32_t *gN = a.n_hist + st.n_off + (long long)t * nb;
         unsigned long long *gG = a.g_hist + st.n_off / (2 * ne) + (long long)t * nc;
-        for (int i = tid; i < nb; i += DENS_T)
+        for (int i = tid; i < nb; i += NT)
             if (s_n[i]) atomicAdd(&gN[i], s_n[i]);
-        for (int i = tid; i < nc; i += DENS_T)
+        for (int i = tid; i < nc; i += NT)
             if (s_gs[i]) atomicAdd(&gG[i], (unsigned long long)s_gs[i]);
         if (vmom) {
             unsigned long long *gV = reinterpret_cast<unsigned long long *>(a.v_hist) + st.n_off / ne +
                                      (long long)t * 2 * nc;
-            for (int i = tid; i < 2 * nc; i += DENS_T)
+            for (int i = tid; i < 2 * nc; i += NT)
                 if (s_v[i]) atomicAdd(&gV[i], s_v[i]);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(DENS_T) k_dens(const Args a)
+{
+    phase_dens(a);
+}
+
+// ---------------------------------------------------------------------------
+// k_run: n_steps whole steps of every stack in one cooperative launch, the
+// phases of each group separated by grid barriers.  All threads of a block work
+// on k_group's and k_dens's phases, the first TPB on the others.  `src_end`:
+// the first step after which no source carrier comes.
+// ---------------------------------------------------------------------------
+template <bool DET, bool DEP, int Q>
+__global__ void __launch_bounds__(32 * GW_MAX, 1) k_run(const Args a, const GroupArgs g, int n_steps, int src_end)
+{
+    uint32_t s = __ldcg(&a.ctl->step);
+    const uint32_t end = s + (uint32_t)n_steps, me = (uint32_t)a.moment_every, ce = (uint32_t)a.compact_every;
+    const bool low = threadIdx.x < TPB;
+    auto failed = [&]() -> bool {            // a decision of the whole block
+        return __syncthreads_or(threadIdx.x == 0 && *(volatile unsigned int *)&a.ctl->status != 0u) != 0;
+    };
+    while (s < end) {
+        uint32_t e = (s / ce + 1) * ce;
+        if (e > s + GROUP_MAX) e = s + GROUP_MAX;
+        if (!DEP && e > (s / me + 1) * me) e = (s / me + 1) * me;
+        if (e > end) e = end;
+        while (s < e) {
+            const bool no_src = s >= (uint32_t)src_end;
+            const Span sp = block_span<DEP>(a, s, (int)(e - s), g.m, no_src);
+            if (sp.len == 0) return;         // (never: the step is this launch's own)
+            phase_group<DET, DEP, Q>(a, g, sp);
+            grid_sync(a);
+            if (low) phase_tail<DET>(a, g, sp, no_src);
+            grid_sync(a);
+            if (failed()) return;
+            s += (uint32_t)sp.len;
+        }
+        if (!DEP && e % me == 0) {
+            phase_dens(a);
+            if (e < end || e % ce == 0) grid_sync(a);
+        }
+        if (e % ce == 0) {
+            if (low) phase_compact<0>(a);
+            if (e < end) grid_sync(a);
         }
     }
 }
@@ -1287,6 +1356,8 @@ cudaError_t group_fits(size_t smem, int threads, bool *ok)
 }
 
 }  // namespace
+
+static cudaError_t configure_run(const Args &a, GroupCfg *c);
 
 cudaError_t configure_group(const Args &a, long long slots, GroupCfg *gc)
 {
@@ -1358,8 +1429,70 @@ cudaError_t configure_group(const Args &a, long long slots, GroupCfg *gc)
         if (od < 1) return cudaSuccess;
         c.grid_dens = sms * std::min(od, 2);
     }
+    e = configure_run(a, &c);
     *gc = c;
-    return cudaSuccess;
+    return e;
+}
+
+// The persistent form's blocks: one per SM, which also have to be enough for a
+// block per stack; shared memory for the largest of its phases.
+template <bool DEP, int Q>
+static cudaError_t run_fits(size_t smem, int threads, bool *ok)
+{
+    int o1 = 0, o2 = 0;
+    cudaError_t e = occupancy(k_run<false, DEP, Q>, smem, &o1, threads);
+    if (e == cudaSuccess) e = occupancy(k_run<true, DEP, Q>, smem, &o2, threads);
+    *ok = e == cudaSuccess && o1 >= 1 && o2 >= 1;
+    return e;
+}
+
+static cudaError_t configure_run(const Args &a, GroupCfg *c)
+{
+    c->run = false;
+    if ((a.flags & PIC_F_WEIGHTS) || c->grid < a.n_stacks) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    // (its static shared memory is larger: a warp or two less)
+    for (int w = c->warps; w >= TPB / 32 && !c->run && e == cudaSuccess; --w) {
+        c->smem_run = std::max({group_smem(a, c->dep, c->quads, w, c->nd, c->nj).total, c->smem_tail, c->smem_dens});
+        c->warps_run = w;
+        if (c->dep) {
+            if (c->quads == 8) e = run_fits<true, 8>(c->smem_run, 32 * w, &c->run);
+            else if (c->quads == 4) e = run_fits<true, 4>(c->smem_run, 32 * w, &c->run);
+            else e = run_fits<true, 2>(c->smem_run, 32 * w, &c->run);
+        } else {
+            if (c->quads == 8) e = run_fits<false, 8>(c->smem_run, 32 * w, &c->run);
+            else if (c->quads == 4) e = run_fits<false, 4>(c->smem_run, 32 * w, &c->run);
+            else e = run_fits<false, 2>(c->smem_run, 32 * w, &c->run);
+        }
+    }
+    return e;
+}
+
+cudaError_t launch_run(const Args &a, const GroupArgs &g, const GroupCfg &c, bool det, int n_steps, int src_end,
+                       cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)c.grid);
+    cfg.blockDim = dim3((unsigned)(32 * c.warps_run));
+    cfg.dynamicSmemBytes = c.smem_run;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+#define PIC_RUN_LAUNCH(DEP, Q)                                                                     \
+    return det ? cudaLaunchKernelEx(&cfg, k_run<true, DEP, Q>, a, g, n_steps, src_end)             \
+               : cudaLaunchKernelEx(&cfg, k_run<false, DEP, Q>, a, g, n_steps, src_end)
+    if (c.dep) {
+        if (c.quads == 8) PIC_RUN_LAUNCH(true, 8);
+        if (c.quads == 4) PIC_RUN_LAUNCH(true, 4);
+        PIC_RUN_LAUNCH(true, 2);
+    }
+    if (c.quads == 8) PIC_RUN_LAUNCH(false, 8);
+    if (c.quads == 4) PIC_RUN_LAUNCH(false, 4);
+    PIC_RUN_LAUNCH(false, 2);
+#undef PIC_RUN_LAUNCH
 }
 
 cudaError_t launch_group(const Args &a, const GroupArgs &g, const GroupCfg &c, bool det, cudaStream_t s)

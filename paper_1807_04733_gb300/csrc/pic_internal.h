@@ -227,7 +227,7 @@ struct GroupArgs {
     uint32_t *abs;               // [n_stacks][GROUP_MAX] carriers removed per step
     uint32_t *bsum, *tsum;       // [GROUP_OPEN][tail blocks] secondaries per block
     GroupRes *res;               // [n_stacks]
-    unsigned int *bar;           // [n_stacks][2] barrier of a stack's tail blocks
+    unsigned int *bar;           // [n_stacks][32] barrier of a stack's tail blocks (a line each)
     const int4 *blk;             // per tail block: stack, index in it, the stack's blocks, the first
     int sub;                     // slots per sub-tile
     int nd, nj;                  // density and removal windows held in shared memory
@@ -238,6 +238,9 @@ struct GroupCfg {
     int m = 0, quads = 0, warps = 0, nd = 0, nj = 0;
     int grid = 0, grid_tail = 0, grid_dens = 0;
     size_t smem = 0, smem_tail = 0, smem_dens = 0;
+    bool run = false;                // the persistent form (one launch for many steps)
+    int warps_run = 0;
+    size_t smem_run = 0;
 };
 
 // reason of the last failure of a call without a context (pic_capi.cu);
@@ -315,6 +318,8 @@ cudaError_t launch_group(const Args &a, const GroupArgs &g, const GroupCfg &gc, 
 cudaError_t launch_tail(const Args &a, const GroupArgs &g, const GroupCfg &gc, bool det,
                         cudaStream_t s);
 cudaError_t launch_dens(const Args &a, const GroupCfg &gc, cudaStream_t s);
+cudaError_t launch_run(const Args &a, const GroupArgs &g, const GroupCfg &gc, bool det, int n_steps,
+                       int src_end, cudaStream_t s);
 cudaError_t launch_mark_base(DevCtl *ctl, cudaStream_t s);
 
 // adjoint replay (pic_adjoint.cu); pass = 1 or 2

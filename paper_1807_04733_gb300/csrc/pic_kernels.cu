@@ -511,37 +511,6 @@ cudaError_t launch_place_fused(const Args &b0, const LaunchCfg &c, bool det, cud
 // from and advanced in device memory, so the launch replays from a graph.
 // ---------------------------------------------------------------------------
 
-// Grid barrier: every block resident (a cooperative launch).  Sense by
-// generation; the wait is bounded in polls, after which the status says
-// PIC_ERR_TIMEOUT and every later barrier of the launch passes at once.
-__device__ __forceinline__ void grid_sync(const Args &a)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        volatile unsigned int *gen = &a.ctl->bar_gen;
-        const unsigned int g = *gen;
-        __threadfence();
-        if (atomicAdd(&a.ctl->bar_count, 1u) == gridDim.x - 1) {
-            a.ctl->bar_count = 0u;           // the next arrivals follow the new generation
-            __threadfence();
-            atomicAdd(&a.ctl->bar_gen, 1u);
-        } else {
-            unsigned int it = 0;
-            while (*gen == g) {
-                if (*(volatile unsigned int *)&a.ctl->status != 0u) break;
-                if (++it > a.spin_limit) {
-                    atomicCAS(&a.ctl->status, 0u, (unsigned int)PIC_ERR_TIMEOUT);
-                    a.ctl->timeout_where = 5u;
-                    break;
-                }
-                if (it > 64) __nanosleep(256);
-            }
-        }
-        __threadfence();
-    }
-    __syncthreads();
-}
-
 // a source half step with carriers in some stack (uniform: device data)
 __device__ __forceinline__ bool any_source(const Args &a, long long h)
 {

@@ -2293,6 +2293,37 @@ __global__ void __launch_bounds__(TPB, 4) k_compact(const Args a)
     phase_compact<ADJ>(a);
 }
 
+// Grid barrier: every block resident (a cooperative launch).  Sense by
+// generation; the wait is bounded in polls, after which the status says
+// PIC_ERR_TIMEOUT and every later barrier of the launch passes at once.
+__device__ __forceinline__ void grid_sync(const Args &a)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        volatile unsigned int *gen = &a.ctl->bar_gen;
+        const unsigned int g = *gen;
+        __threadfence();
+        if (atomicAdd(&a.ctl->bar_count, 1u) == gridDim.x - 1) {
+            a.ctl->bar_count = 0u;           // the next arrivals follow the new generation
+            __threadfence();
+            atomicAdd(&a.ctl->bar_gen, 1u);
+        } else {
+            unsigned int it = 0;
+            while (*gen == g) {
+                if (*(volatile unsigned int *)&a.ctl->status != 0u) break;
+                if (++it > a.spin_limit) {
+                    atomicCAS(&a.ctl->status, 0u, (unsigned int)PIC_ERR_TIMEOUT);
+                    a.ctl->timeout_where = 5u;
+                    break;
+                }
+                if (it > 64) __nanosleep(256);
+            }
+        }
+        __threadfence();
+    }
+    __syncthreads();
+}
+
 // ---------------------------------------------------------------------------
 // host-side launch-configuration helpers shared by the forward and adjoint
 // translation units
