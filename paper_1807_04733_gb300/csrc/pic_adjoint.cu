@@ -24,6 +24,8 @@
 // streaming pass runs integer adds instead of double-precision arithmetic.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "pic_step.cuh"
 
 namespace pic {
@@ -223,10 +225,12 @@ cudaError_t launch_slow_adj(const Args &a0, const LaunchCfg &c, int pass, bool d
 }
 
 cudaError_t launch_inject_adj(const Args &a, const LaunchCfg &c, int pass, int half, bool deposit,
-                              cudaStream_t s)
+                              long long n, cudaStream_t s)
 {
-    if (pass == 1) k_inject<1><<<c.grid_inject, TPB, 0, s>>>(a, half, deposit ? 1 : 0);
-    else k_inject<2><<<c.grid_inject, TPB, 0, s>>>(a, half, deposit ? 1 : 0);
+    // as many blocks as the half step's n carriers fill
+    const int g = (int)std::min<long long>(c.grid_inject, std::max<long long>(1, (n + TPB - 1) / TPB));
+    if (pass == 1) k_inject<1><<<g, TPB, 0, s>>>(a, half, deposit ? 1 : 0);
+    else k_inject<2><<<g, TPB, 0, s>>>(a, half, deposit ? 1 : 0);
     return cudaGetLastError();
 }
 

@@ -1945,19 +1945,19 @@ pic_status pic_grad(pic_ctx *c, const float *grad_n, const float *grad_J, double
         // the steps of the forward run, in the same order
         for (int step = 0; step < c->step && e == cudaSuccess; ++step) {
             a.step = (uint32_t)step;
-            bool inj0 = false, inj1 = false;
+            long long inj0 = 0, inj1 = 0;
             for (const HostStack &h : c->hs) {
-                inj0 = inj0 || h.inj[2 * (size_t)step] > 0;
-                inj1 = inj1 || h.inj[2 * (size_t)step + 1] > 0;
+                inj0 += h.inj[2 * (size_t)step];
+                inj1 += h.inj[2 * (size_t)step + 1];
             }
             const bool dep = ((step + 1) % c->p.moment_every) == 0;
-            if (inj0) e = timed(c, 7, [&] { return launch_inject_adj(a, lc, pass, 0, false, st); });
+            if (inj0) e = timed(c, 7, [&] { return launch_inject_adj(a, lc, pass, 0, false, inj0, st); });
             if (e == cudaSuccess)
                 e = timed(c, 5, [&] { return launch_fast_adj(a, lc, pass, det, dep, st); });
             if (e == cudaSuccess)
                 e = timed(c, 6, [&] { return launch_slow_adj(a, lc, pass, det, dep, st); });
             if (e == cudaSuccess && inj1)
-                e = timed(c, 7, [&] { return launch_inject_adj(a, lc, pass, 1, dep, st); });
+                e = timed(c, 7, [&] { return launch_inject_adj(a, lc, pass, 1, dep, inj1, st); });
             if (e == cudaSuccess && ((step + 1) % c->p.compact_every) == 0)
                 e = timed(c, 7, [&] { return launch_compact_adj(a, lc, pass, st); });
         }

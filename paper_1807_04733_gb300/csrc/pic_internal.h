@@ -325,7 +325,7 @@ cudaError_t launch_mark_base(DevCtl *ctl, cudaStream_t s);
 // adjoint replay (pic_adjoint.cu); pass = 1 or 2
 cudaError_t configure_adjoint(const Args &a, int pass, LaunchCfg *cfg);
 cudaError_t launch_inject_adj(const Args &a, const LaunchCfg &c, int pass, int half,
-                              bool deposit, cudaStream_t s);
+                              bool deposit, long long n, cudaStream_t s);
 cudaError_t launch_fast_adj(const Args &a, const LaunchCfg &c, int pass, bool deterministic,
                             bool deposit, cudaStream_t s);
 cudaError_t launch_slow_adj(const Args &a, const LaunchCfg &c, int pass, bool deterministic,

@@ -1547,8 +1547,8 @@ __device__ __forceinline__ void phase_event(const Args &a)
     };
 
     if (i0 < i1) {
-        const int s_first = stack_of(s_tpref, a.n_stacks, tile_of(i0));
-        const int s_last = stack_of(s_tpref, a.n_stacks, tile_of(i1 - 1));
+        const int s_first = a.n_stacks == 1 ? 0 : stack_of(s_tpref, a.n_stacks, tile_of(i0));
+        const int s_last = a.n_stacks == 1 ? 0 : stack_of(s_tpref, a.n_stacks, tile_of(i1 - 1));
         long long lo = i0;
         for (int s = s_first; s <= s_last; ++s) {
             if (s_tpref[s + 1] == s_tpref[s]) continue;       // a stack with no tiles
@@ -2023,9 +2023,13 @@ __device__ __forceinline__ void phase_inject(const Args &a, int half, int deposi
         const uint32_t cy = (uint32_t)(id >> 32) | ((uint32_t)(a.stack_base + s) << 16);
         const uint4 r0 = philox_rk(make_uint4((uint32_t)id, cy, step, SUB_INJ + 0), a);
         const uint4 r1 = philox_rk(make_uint4((uint32_t)id, cy, step, SUB_INJ + 1), a);
-        int i = 0;
+        // the first entry whose threshold lies above the word, or the last
         const uint32_t *thr = a.cdf_thr + st.cdf_off;
-        while (i < st.n_cdf - 1 && !(r0.x < thr[i])) ++i;
+        int i = 0;
+        for (int hi = st.n_cdf - 1; i < hi;) {
+            const int mid = (i + hi) >> 1;
+            if (r0.x < thr[mid]) hi = mid; else i = mid + 1;
+        }
         const int cell = a.cdf_cell[st.cdf_off + i];
         const float z = __fmul_rn(__fadd_rn((float)cell, unit_of(r0.y)), a.dz);
         const uint32_t sg = r0.z < st.up_thr ? 0u : 1u;
@@ -2047,7 +2051,12 @@ __device__ __forceinline__ void phase_inject(const Args &a, int half, int deposi
             __float_as_uint(mu_of(r1.x)),
             k | (sg << 8) | (layer << 9) | (1u << 13) | ((uint32_t)(id >> 32) << 21));
         a.id[cur][d] = (uint32_t)id;
-        atomicAdd(&s_q[s], (unsigned long long)k);
+        {
+            // the quanta of the warp's carriers of one stack at once
+            const unsigned int same = __match_any_sync(__activemask(), s);
+            const uint32_t q = __reduce_add_sync(same, k);
+            if ((int)(threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(&s_q[s], (unsigned long long)q);
+        }
         uint32_t wq = 1u << 20;
         if (!ADJ && a.w[0]) {
             // weight p/q of the birth cell and bin (Eq. PIC), 2^-20 units
