@@ -183,6 +183,21 @@ __host__ __device__ inline GroupSmem group_smem(const Args &a, bool dep, int qua
     return o;
 }
 
+// Adds a block's nb bins (an even number) to those in memory, two at a time: the
+// sums stay below 2^32, so a pair of bins is one 64-bit number without a carry
+// between them, and the additions at the L2 are what this takes.  Every block
+// starts at bins of its own.
+__device__ __forceinline__ void flush_bins(uint32_t *dst, const uint32_t *src, int nb)
+{
+    const int np = nb / 2, rot = (int)((long long)blockIdx.x * np / (int)gridDim.x) & ~15;
+    unsigned long long *d = reinterpret_cast<unsigned long long *>(dst);
+    for (int i = threadIdx.x; i < np; i += (int)blockDim.x) {
+        const int b = i + rot < np ? i + rot : i + rot - np;
+        const uint32_t lo = src[2 * b], hi = src[2 * b + 1];
+        if (lo | hi) atomicAdd(&d[b], (unsigned long long)lo | ((unsigned long long)hi << 32));
+    }
+}
+
 // ---------------------------------------------------------------------------
 // k_group.  A lane owns 4 Q consecutive slots of its warp's sub-tile of 128 Q
 // slots.  The depth is kept in the direction of flight: z' = z for a carrier
@@ -663,10 +678,7 @@ __device__ __forceinline__ void phase_group(const Args &a, const GroupArgs &g, c
             unsigned long long *gV = reinterpret_cast<unsigned long long *>(a.v_hist) + st.n_off / ne +
                                      (long long)tj0 * 2 * nc;
             for (int h = 0; h < ndep; ++h) {
-                for (int i = tid; i < nb; i += NT) {
-                    const uint32_t v = s_n[h * hb + i];
-                    if (v) atomicAdd(&gN[(long long)h * nb + i], v);
-                }
+                flush_bins(gN + (long long)h * nb, s_n + h * hb, nb);
                 for (int i = tid; i < nc; i += NT) {
                     const uint32_t v = s_gs[h * nc + i];
                     if (v) atomicAdd(&gG[(long long)h * nc + i], (unsigned long long)v);
@@ -1276,8 +1288,7 @@ __device__ __forceinline__ void phase_dens(const Args &a)
         __syncthreads();
         uint32_t *gN = a.n_hist + st.n_off + (long long)t * nb;
         unsigned long long *gG = a.g_hist + st.n_off / (2 * ne) + (long long)t * nc;
-        for (int i = tid; i < nb; i += NT)
-            if (s_n[i]) atomicAdd(&gN[i], s_n[i]);
+        flush_bins(gN, s_n, nb);
         for (int i = tid; i < nc; i += NT)
             if (s_gs[i]) atomicAdd(&gG[i], (unsigned long long)s_gs[i]);
         if (vmom) {
