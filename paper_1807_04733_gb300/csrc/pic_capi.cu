@@ -130,6 +130,7 @@ struct pic_ctx {
     // tail blocks' shares
     GroupCfg gc;
     GroupArgs ga{};
+    uint2 *d_glist = nullptr;        // lists of steps 4 to 7 of a group
     uint16_t *d_gcnt = nullptr;
     uint32_t *d_gabs = nullptr, *d_gsum = nullptr;
     GroupRes *d_gres = nullptr;
@@ -394,7 +395,7 @@ void free_all(pic_ctx *c)
     release(c->d_w[0]); release(c->d_w[1]); release(c->d_wcell); release(c->d_wbin);
     release(c->d_kthr); release(c->d_nhw); release(c->d_bdw); release(c->d_Jw); release(c->d_hnow_w);
     release(c->d_ctl);
-    release(c->d_gcnt); release(c->d_gabs); release(c->d_gsum); release(c->d_gres); release(c->d_gbar);
+    release(c->d_glist); release(c->d_gcnt); release(c->d_gabs); release(c->d_gsum); release(c->d_gres); release(c->d_gbar);
     release(c->d_gblk);
     Replay &r = c->rp;
     for (int b = 0; b < 2; ++b) {
@@ -776,8 +777,13 @@ pic_status pic_init(pic_ctx **out, const pic_params *p, const pic_stack_desc *st
         };
         share(gt);
         if (c->gc.run) share(gr);
-        // the lists of the four steps: one 8-byte record per slot and step, in
-        // the buffers of the single steps' staged and queued records
+        // the lists of the steps: one 8-byte record per slot and step, in the
+        // buffers of the single steps' staged and queued records, and more for
+        // groups of more than four steps
+        if (e == cudaSuccess && c->gc.m > GROUP_OPEN_LARGE)
+            e = dalloc(&c->d_glist, (size_t)(GROUP_OPEN - GROUP_OPEN_LARGE) * c->total_slots);
+        g.list[2] = c->d_glist;
+        g.list[3] = c->d_glist ? c->d_glist + 2 * c->total_slots : nullptr;
         g.list[0] = reinterpret_cast<uint2 *>(c->d_stage);
         g.list[1] = reinterpret_cast<uint2 *>(c->d_qrec);
         g.list_n = c->total_slots;
@@ -1023,7 +1029,7 @@ cudaError_t enqueue_range(pic_ctx *c, const Args &a0, int s, int e, const unsign
     cudaError_t r = cudaSuccess;
     for (int o = s; o < e && r == cudaSuccess; o += g.m) {
         g.off = o;
-        g.m = std::min(gc.m, e - o);
+        g.m = group_part(e - o, gc.m);
         g.no_src = base ? !src : !any_source(c, o, e - o);
         r = timed(c, gc.dep ? 2 : 1, [&] { return launch_group(a, g, gc, det, st); });
         if (r == cudaSuccess) r = timed(c, 4, [&] { return launch_tail(a, g, gc, det, st); });

@@ -133,7 +133,8 @@ __device__ __forceinline__ Span group_span(const Args &a, uint32_t s0, int span,
 
 __device__ __forceinline__ uint2 *list_of(const GroupArgs &g, int j)
 {
-    return (j < 2 ? g.list[0] : g.list[1]) + (j & 1) * g.list_n;
+    uint2 *p = j < 4 ? (j < 2 ? g.list[0] : g.list[1]) : (j < 6 ? g.list[2] : g.list[3]);
+    return p + (j & 1) * g.list_n;
 }
 
 // A slot's test word: the upper half of its threshold, and the edge ahead as
@@ -1327,7 +1328,7 @@ __global__ void __launch_bounds__(32 * GW_MAX, 1) k_run(const Args a, const Grou
         if (e > end) e = end;
         while (s < e) {
             const bool no_src = s >= (uint32_t)src_end;
-            const Span sp = block_span<DEP>(a, s, (int)(e - s), g.m, no_src);
+            const Span sp = block_span<DEP>(a, s, (int)(e - s), group_part((int)(e - s), g.m), no_src);
             if (sp.len == 0) return;         // (never: the step is this launch's own)
             phase_group<DET, DEP, Q>(a, g, sp);
             grid_sync(a);
@@ -1384,7 +1385,7 @@ cudaError_t configure_group(const Args &a, long long slots, GroupCfg *gc)
     // the edges have to do as half-precision numbers
     if (a.dz * (float)a.gbin_max > 32768.f || a.dz < 1.f / 1024.f) return cudaSuccess;
     GroupCfg c;
-    c.dep = me < GROUP_OPEN && !wts;
+    c.dep = me < GROUP_DEP_EVERY && !wts;
     // Slots per sub-tile: 1024, so that the 2 % of eventful carriers fill most of
     // a warp (41.5 ms for 50 steps of 4e8 carriers; 52.9 with 512); 512 beside
     // the density histograms, which leave room for too few warps otherwise
@@ -1396,13 +1397,14 @@ cudaError_t configure_group(const Args &a, long long slots, GroupCfg *gc)
 #ifdef PIC_GROUP_Q
     if (c.quads > PIC_GROUP_Q) c.quads = PIC_GROUP_Q;
 #endif
-    for (int m = GROUP_OPEN; m >= 1 && !c.ok; --m) {
+    for (int m = slots <= GROUP_LIST_SLOTS ? GROUP_OPEN : GROUP_OPEN_LARGE; m >= 1 && !c.ok; --m) {
         const int nd = c.dep ? (me - 1 + m) / me : 0;
         const int nj = c.dep ? (me + m - 2) / me + 1 : 1;
         for (int w = GW_MAX; w >= 4; --w) {
             const GroupSmem o = group_smem(a, c.dep, c.quads, w, nd, nj);
             if (o.total > cap) continue;
-            if (w < (c.quads == 8 ? 6 : c.quads == 4 ? 8 : 12) && m > 1) break;      // too few warps: fewer windows
+            // too few warps beside the histograms: fewer windows
+            if (m > 1 && w < (c.quads == 8 ? 6 : c.quads == 4 ? (m > GROUP_OPEN_LARGE ? 14 : 8) : 12)) break;
             bool ok = false;
             if (c.dep) {
                 if (c.quads == 8) e = group_fits<true, 8>(o.total, 32 * w, &ok);

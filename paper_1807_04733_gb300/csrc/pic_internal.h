@@ -205,7 +205,15 @@ struct Args {            // everything a kernel needs, passed by value
 };
 
 // Groups of time steps run in one pass over memory (pic_group.cu).
-constexpr int GROUP_OPEN = 4;    // most steps of a group that may create secondaries
+// Most steps of a group that may create secondaries: eight where the launches and
+// barriers of a group count (a run of 500 steps from 1e5 carriers 8.2 -> 7.6 ms);
+// four in contexts of more than GROUP_LIST_SLOTS, where the new carriers, which
+// draw their test words one by one, would cost more than the passes over the others
+// save (500 steps from 2e7 carriers 85.0 against 86.5 ms with eight) and the record
+// lists of more steps would need memory of their own.
+constexpr int GROUP_OPEN = 8, GROUP_OPEN_LARGE = 4;
+constexpr long long GROUP_LIST_SLOTS = 8ll << 20;
+constexpr int GROUP_DEP_EVERY = 4;   // densities inside the groups if taken more often than this
 constexpr int GROUP_MAX = 64;    // most steps of a closed group
 constexpr int GROUP_SUB_MIN = 256;   // fewest slots of a warp's sub-tile
 
@@ -220,7 +228,7 @@ struct GroupArgs {
     const unsigned int *base;    // off and end count from *base (graph replay); null: from 0
     // new secondaries (depth, k | layer | gen | position) of step j of the
     // group: list_n entries at list[j / 2] + (j % 2) list_n
-    uint2 *list[2];
+    uint2 *list[GROUP_OPEN / 2];
     long long list_n;
     uint16_t *cnt;               // [GROUP_OPEN][cnt_n] secondaries per sub-tile
     long long cnt_n;
@@ -232,6 +240,16 @@ struct GroupArgs {
     int sub;                     // slots per sub-tile
     int nd, nj;                  // density and removal windows held in shared memory
 };
+
+// Steps of the next group of a range of n: equal parts of at most m.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int group_part(int n, int m)
+{
+    const int parts = (n + m - 1) / m;
+    return (n + parts - 1) / parts;
+}
 
 struct GroupCfg {
     bool ok = false, dep = false;    // dep: densities deposited inside the group
