@@ -99,6 +99,11 @@ struct pic_ctx {
     int64_t total_slots = 0, nh_total = 0, J_total = 0;
     int n_status = 0;                // queue counts allocated
     size_t n_words = 0;              // look-back words allocated
+    // what reading calls bring to the host, written by the device: a member
+    // of this structure where the device reaches ordinary host memory (mapped
+    // memory takes a third of a millisecond to allocate), else mapped memory
+    HostRead h_own{};
+    HostRead *h_read = nullptr, *h_read_dev = nullptr;
     Args args{};
     LaunchCfg lc{};
     int step = 0;
@@ -395,6 +400,8 @@ void free_all(pic_ctx *c)
     release(c->d_w[0]); release(c->d_w[1]); release(c->d_wcell); release(c->d_wbin);
     release(c->d_kthr); release(c->d_nhw); release(c->d_bdw); release(c->d_Jw); release(c->d_hnow_w);
     release(c->d_ctl);
+    if (c->h_read && c->h_read != &c->h_own) cudaFreeHost(c->h_read);
+    c->h_read = nullptr;
     release(c->d_glist); release(c->d_gcnt); release(c->d_gabs); release(c->d_gsum); release(c->d_gres); release(c->d_gbar);
     release(c->d_gblk);
     Replay &r = c->rp;
@@ -446,19 +453,62 @@ int source_end(const pic_ctx *c)
     return e;
 }
 
+pic_status status_result(pic_ctx *c, unsigned int status)
+{
+    if (status != 0) {
+        const pic_status s = (pic_status)status;
+        return fail(c, s, s == PIC_ERR_TIMEOUT    ? "a bounded device wait ran out"
+                          : s == PIC_ERR_CAPACITY ? "capacity exceeded in strict mode"
+                                                  : "the adjoint replay did not reproduce the forward run");
+    }
+    return PIC_OK;
+}
+
 pic_status device_status(pic_ctx *c)
 {
     DevCtl h{};
     cudaError_t e = cudaMemcpyAsync(&h, c->d_ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "device status");
-    if (h.status != 0) {
-        const pic_status s = (pic_status)h.status;
-        return fail(c, s, s == PIC_ERR_TIMEOUT    ? "a bounded device wait ran out"
-                          : s == PIC_ERR_CAPACITY ? "capacity exceeded in strict mode"
-                                                  : "the adjoint replay did not reproduce the forward run");
+    return status_result(c, h.status);
+}
+
+bool on_device(const void *p)
+{
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
     }
-    return PIC_OK;
+    return at.type == cudaMemoryTypeDevice;
+}
+
+// Ends a reading call: copies n_words and j_words words (destinations in host or
+// device memory; null: none), brings the stack's counters and the device status
+// to the host and waits.  What stays on the device goes with the counters in
+// one launch; they come by mapped host memory, where a copy of each from
+// pageable memory took most of a small call's time.
+pic_status read_out(pic_ctx *c, int stack, const uint32_t *n_src, void *n_dst, size_t n_words,
+                    const uint32_t *j_src, void *j_dst, size_t j_words, DevCounters *hc, const char *where)
+{
+    cudaError_t e = cudaSuccess;
+    // (a copy engine is as good for large ones)
+    const size_t most = 1u << 20;
+    const bool nk = n_dst && n_words && n_words <= most && on_device(n_dst);
+    const bool jk = j_dst && j_words && j_words <= most && on_device(j_dst);
+    if (n_dst && n_words && !nk) e = cudaMemcpyAsync(n_dst, n_src, 4 * n_words, cudaMemcpyDefault, c->stream);
+    if (e == cudaSuccess && j_dst && j_words && !jk)
+        e = cudaMemcpyAsync(j_dst, j_src, 4 * j_words, cudaMemcpyDefault, c->stream);
+    if (e == cudaSuccess)
+        e = launch_read(c->d_cnt + stack, c->d_ctl, c->h_read_dev, n_src, static_cast<uint32_t *>(n_dst),
+                        nk ? (long long)n_words : 0, j_src, static_cast<uint32_t *>(j_dst),
+                        jk ? (long long)j_words : 0, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, where);
+    HostRead r;
+    std::memcpy(&r, const_cast<const HostRead *>(c->h_read), sizeof(r));
+    if (hc) *hc = r.cnt;
+    return status_result(c, r.status);
 }
 
 }  // namespace
@@ -658,6 +708,15 @@ pic_status pic_init(pic_ctx **out, const pic_params *p, const pic_stack_desc *st
     ALLOC(c->d_hnow, (size_t)n_stacks * 2 * (c->ncm + 1));
     ALLOC(c->d_cnt, n_stacks);
     ALLOC(c->d_ctl, 1);
+    int dev_id = 0, pageable = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev_id);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, dev_id);
+    if (e == cudaSuccess && pageable) {
+        c->h_read = c->h_read_dev = &c->h_own;
+    } else {
+        if (e == cudaSuccess) e = cudaHostAlloc((void **)&c->h_read, sizeof(HostRead), cudaHostAllocMapped);
+        if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&c->h_read_dev, c->h_read, 0);
+    }
 #undef ALLOC
     if (e != cudaSuccess) {
         g_init_error = std::string("device allocation: ") + cudaGetErrorString(e);
@@ -1486,12 +1545,9 @@ pic_status pic_moments(pic_ctx *c, int stack, uint32_t *n_dev, int32_t *J_dev, p
     if (e != cudaSuccess) return cuda_fail(c, e, "pic_moments fluxes");
     const size_t nn = (size_t)h.n_out * 2 * c->p.n_e * h.n_cells;
     const size_t nj = (size_t)h.n_out * 2 * (h.n_cells + 1);
-    if (n_dev && nn) e = cudaMemcpyAsync(n_dev, c->d_nh + d.n_off, 4 * nn, cudaMemcpyDeviceToDevice, c->stream);
-    if (e == cudaSuccess && J_dev && nj) e = cudaMemcpyAsync(J_dev, c->d_J + d.J_off, 4 * nj, cudaMemcpyDeviceToDevice, c->stream);
     DevCounters hc{};
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&hc, c->d_cnt + stack, sizeof(DevCounters), cudaMemcpyDeviceToHost, c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "pic_moments copy");
-    const pic_status st = device_status(c);
+    const pic_status st = read_out(c, stack, c->d_nh + d.n_off, n_dev, nn, reinterpret_cast<const uint32_t *>(c->d_J + d.J_off),
+                                   J_dev, nj, &hc, "pic_moments copy");
     if (led) {
         static_assert(sizeof(pic_ledger) == sizeof(unsigned long long) * LEDGER_N, "ledger layout");
         std::memcpy(led, hc.led, sizeof(pic_ledger));
@@ -1511,14 +1567,10 @@ pic_status pic_moment_window(pic_ctx *c, int stack, int window, uint32_t *n_out,
     if (e != cudaSuccess) return cuda_fail(c, e, "pic_moment_window fluxes");
     const size_t nn = (size_t)2 * c->p.n_e * h.n_cells;
     const size_t nj = (size_t)2 * (h.n_cells + 1);
-    // the buffers may be host or device memory (unified addressing)
-    if (n_out) e = cudaMemcpyAsync(n_out, c->d_nh + d.n_off + (size_t)window * nn, 4 * nn, cudaMemcpyDefault, c->stream);
-    if (e == cudaSuccess && J_out)
-        e = cudaMemcpyAsync(J_out, c->d_J + d.J_off + (size_t)window * nj, 4 * nj, cudaMemcpyDefault, c->stream);
     DevCounters hc{};
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&hc, c->d_cnt + stack, sizeof(DevCounters), cudaMemcpyDeviceToHost, c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "pic_moment_window copy");
-    const pic_status st = device_status(c);
+    const pic_status st = read_out(c, stack, c->d_nh + d.n_off + (size_t)window * nn, n_out, nn,
+                                   reinterpret_cast<const uint32_t *>(c->d_J + d.J_off + (size_t)window * nj), J_out, nj,
+                                   &hc, "pic_moment_window copy");
     if (led) std::memcpy(led, hc.led, sizeof(pic_ledger));
     return st;
 }

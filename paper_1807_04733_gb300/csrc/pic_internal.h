@@ -116,6 +116,11 @@ struct DevCtl {
     unsigned int ticket;     // next tile of the compaction
 };
 
+struct HostRead {        // in mapped host memory: what a reading call returns
+    DevCounters cnt;
+    unsigned int status;
+};
+
 struct Args {            // everything a kernel needs, passed by value
     const DevStack *stacks;
     int n_stacks;
@@ -313,6 +318,9 @@ cudaError_t launch_flux(const Args &a, int w0, int w1, int w_now, const int32_t 
 // the weighted fluxes Jw from nhw, bdw (and `now` [stack][2][ncm+1] int64)
 cudaError_t launch_flux_w(const Args &a, int w0, int w1, int w_now, const long long *now, int ncm,
                           cudaStream_t st);
+cudaError_t launch_read(const DevCounters *cnt, const DevCtl *ctl, HostRead *out, const uint32_t *n_src,
+                        uint32_t *n_dst, long long n_words, const uint32_t *j_src, uint32_t *j_dst,
+                        long long j_words, cudaStream_t s);
 // set the device step counter read by graph-replayed steps
 cudaError_t launch_set_step(DevCtl *ctl, unsigned int step, cudaStream_t s);
 // the persistent kernel: n_steps whole steps of every stack in one cooperative

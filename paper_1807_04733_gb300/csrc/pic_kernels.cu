@@ -248,6 +248,35 @@ __global__ void __launch_bounds__(TPB) k_wdep(const Args a)
     phase_wdep<SM>(a, a.step_dev ? __ldcg(a.step_dev) - 1u : a.step);
 }
 
+// What a reading call takes to the host: a stack's counters and the device
+// status, into mapped host memory; and two device-to-device copies (either may
+// be empty), in the same launch.
+__global__ void __launch_bounds__(TPB) k_read(const DevCounters *cnt, const DevCtl *ctl, HostRead *out,
+                                              const uint32_t *n_src, uint32_t *n_dst, long long n_words,
+                                              const uint32_t *j_src, uint32_t *j_dst, long long j_words)
+{
+    const long long i0 = (long long)blockIdx.x * TPB + threadIdx.x, step = (long long)gridDim.x * TPB;
+    for (long long i = i0; i < n_words; i += step) n_dst[i] = n_src[i];
+    for (long long i = i0; i < j_words; i += step) j_dst[i] = j_src[i];
+    constexpr int W = (int)(sizeof(DevCounters) / 8);
+    if (blockIdx.x == 0) {
+        if (threadIdx.x < W)
+            reinterpret_cast<unsigned long long *>(&out->cnt)[threadIdx.x] =
+                reinterpret_cast<const unsigned long long *>(cnt)[threadIdx.x];
+        if (threadIdx.x == W) out->status = ctl->status;
+    }
+}
+
+cudaError_t launch_read(const DevCounters *cnt, const DevCtl *ctl, HostRead *out, const uint32_t *n_src,
+                        uint32_t *n_dst, long long n_words, const uint32_t *j_src, uint32_t *j_dst,
+                        long long j_words, cudaStream_t s)
+{
+    const long long w = std::max(n_words, j_words);
+    const int g = (int)std::max<long long>(1, std::min<long long>((w + 2 * TPB - 1) / (2 * TPB), 256));
+    k_read<<<g, TPB, 0, s>>>(cnt, ctl, out, n_src, n_dst, n_words, j_src, j_dst, j_words);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_flux_w(const Args &a, int w0, int w1, int w_now, const long long *now, int ncm,
                           cudaStream_t st)
 {
