@@ -741,14 +741,19 @@ __device__ __forceinline__ void agg_sum(unsigned long long *p, uint32_t v)
     if ((int)(threadIdx.x & 31) == __ffs(m) - 1) atomicAdd(p, (unsigned long long)t);
 }
 
-// Barrier of the stack's nb blocks (all resident: a cooperative launch): one
+// Barrier of the stack's nb blocks (all resident: a cooperative launch) in two
+// halves, between which a block works on what needs no other block: one
 // counter that only grows, `target` the arrivals that end this barrier.  One
 // trip to memory to arrive, then polls; bounded in polls.
-__device__ __forceinline__ void stack_sync(const Args &a, unsigned int *bar, unsigned int target)
+__device__ __forceinline__ void stack_arrive(unsigned int *bar)
 {
     cta_sync();
+    if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+}
+
+__device__ __forceinline__ void stack_wait(const Args &a, unsigned int *bar, unsigned int target)
+{
     if (threadIdx.x == 0) {
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
         unsigned int it = 0, v;
         for (;;) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
@@ -764,6 +769,12 @@ __device__ __forceinline__ void stack_sync(const Args &a, unsigned int *bar, uns
     }
     cta_sync();
 }
+
+struct TailChild {                   // a secondary before its slot is known
+    float z, mu, zb, v;              // depth and direction after its half flight; where it was born; speed
+    uint32_t pk, pslot;              // packed word without the id; the parent's slot
+    uint32_t hits, trans, trunc;
+};
 
 struct TailStack {                   // what a tail block keeps of its stack
     const DevStack *st;
@@ -909,7 +920,74 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
         }
         cta_sync();
         if (tid < sp.len) g.bsum[(long long)(b0 + ib) * GROUP_OPEN + tid] = s_tot[tid];
-        stack_sync(a, bar, bar_t += (unsigned int)nbk);
+        stack_arrive(bar);
+
+        // A secondary from its record; it depends on nothing but the record.
+        auto make = [&](uint32_t step, const uint2 rec, long long pslot) -> TailChild {
+            const int ks = (int)(rec.y & 0xFFu);
+            int layer = (int)((rec.y >> 8) & 0xFu);
+            const uint32_t g0 = (rec.y >> 12) & 0xFFu, gen = g0 < 255u ? g0 + 1u : 255u;
+            const uint4 y = philox_rk(make_uint4((uint32_t)pslot, x.ctr_hi, step, SUB_SEC), a);
+            const int sg = y.x < s_p0[layer] ? 0 : 1;
+            TailChild c;
+            c.zb = __uint_as_float(rec.x);
+            c.z = c.zb;
+            c.mu = mu_of(y.y);
+            float lo = s_edge[layer], hi = s_edge[layer + 1];
+            TabEnt e = s_ent[(layer * 2 + sg) * x.ne + (ks - 1)];
+            Tally tq{};
+            flight<DET>(a, S, c.z, c.mu, layer, e, lo, hi, sg, ks, half, (uint32_t)pslot, x.ctr_hi, step,
+                        SUB_SIF, tq);
+            c.v = e.v;
+            c.pk = (uint32_t)ks | ((uint32_t)sg << 8) | ((uint32_t)layer << 9) | (gen << 13);
+            c.pslot = (uint32_t)pslot;
+            c.hits = tq.hits;
+            c.trans = tq.trans;
+            c.trunc = tq.trunc;
+            return c;
+        };
+        // The records of step j in sub-tiles [p0, p0 + np) of this block: a prefix
+        // of their counts in s_pre; the number of records.
+        auto prefix = [&](int j, long long p0, int np) -> int {
+            int c[TAIL_PIECE / TPB], sum = 0;
+#pragma unroll
+            for (int q = 0; q < TAIL_PIECE / TPB; ++q) {
+                const int i = tid * (TAIL_PIECE / TPB) + q;
+                c[q] = i < np ? (int)cnt[j * g.cnt_n + p0 + i] : 0;
+                sum += c[q];
+            }
+            int excl;
+            const int tot = block_scan(sum, excl, s_w);
+            if (tot == 0) return 0;
+#pragma unroll
+            for (int q = 0; q < TAIL_PIECE / TPB; ++q) {
+                s_pre[tid * (TAIL_PIECE / TPB) + q] = (uint32_t)excl;
+                excl += c[q];
+            }
+            cta_sync();
+            return tot;
+        };
+        auto record = [&](int j, long long p0, int r) -> TailChild {
+            int lo = 0, hi = TAIL_PIECE - 1;         // last sub-tile with prefix <= r
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (s_pre[mid] <= (uint32_t)r) lo = mid; else hi = mid - 1;
+            }
+            const long long sl0 = (p0 + lo) * g.sub;
+            const uint2 rec = __ldcg(&(list_of(g, j) + st.base)[sl0 + (r - (int)s_pre[lo])]);
+            return make(sp.s0 + (uint32_t)j, rec, sl0 + (rec.y >> 20));
+        };
+        // The first TPB secondaries of the next step (most often all) are made
+        // while the block waits for the others at the barrier before it.
+        const int np0 = (int)(u1 - u0 < TAIL_PIECE ? u1 - u0 : TAIL_PIECE);
+        TailChild ch{};
+        int tot0 = 0;
+        auto prepare = [&](int j) {
+            tot0 = prefix(j, u0, np0);
+            if (tid < tot0) ch = record(j, u0, tid);
+        };
+        prepare(0);
+        stack_wait(a, bar, bar_t += (unsigned int)nbk);
         if (tid < GROUP_OPEN) s_tot[tid] = 0u;
         cta_sync();
         for (int i = tid; i < nbk * sp.len; i += TPB) {
@@ -937,13 +1015,26 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
             const long long L = nsl + i0 - n0;
             const long long x0 = L * ib / nbk, x1 = L * (ib + 1) / nbk;
             uint32_t mine = 0;
+            float z_next = 0.f;              // the next carrier's record, asked for one round ahead
+            uint2 mp_next = make_uint2(0u, 0u);
+            auto ask = [&](long long xi) {
+                if (xi < x1 && n0 + xi < nsl) {
+                    z_next = __ldcg(x.Z + n0 + xi);
+                    mp_next = __ldcg(reinterpret_cast<const uint2 *>(x.MU + 2 * (n0 + xi)));
+                }
+            };
+            ask(x0 + tid);
 #pragma unroll 1
             for (long long xi = x0 + tid; xi < x1; xi += TPB) {
                 const long long slot = n0 + xi;
-                if (slot >= nsl)
+                float z = z_next;
+                uint2 mp = mp_next;
+                ask(xi + TPB);
+                if (slot >= nsl) {
                     tail_source(a, x, step, t, nid + (unsigned long long)(slot - nsl), slot, false, q_src, w_src);
-                float z = __ldcg(x.Z + slot);
-                const uint2 mp = __ldcg(reinterpret_cast<const uint2 *>(x.MU + 2 * slot));
+                    z = __ldcg(x.Z + slot);
+                    mp = __ldcg(reinterpret_cast<const uint2 *>(x.MU + 2 * slot));
+                }
                 float mu = __uint_as_float(mp.x);
                 uint32_t pk = mp.y;
                 uint2 rec = make_uint2(0u, 0u);
@@ -1024,7 +1115,8 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
                 if (lane == 0 && mine) atomicAdd(&s_tt[0], mine);
                 cta_sync();
                 if (tid == 0) g.tsum[(long long)(b0 + ib) * GROUP_OPEN + j] = s_tt[0];
-                stack_sync(a, bar, bar_t += (unsigned int)nbk);
+                stack_arrive(bar);
+                stack_wait(a, bar, bar_t += (unsigned int)nbk);
                 if (tid == 0) s_tt[0] = 0u;
                 cta_sync();
                 for (int b = tid; b < nbk; b += TPB) {
@@ -1050,74 +1142,44 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
             const long long room = st.cap - nsl;
             const long long total = (long long)s_tot[j] + tail_tot;
             const long long kept = total < room ? total : (room > 0 ? room : 0);
-            auto place = [&](const uint2 rec, long long pslot, long long rank) {
-                const int ks = (int)(rec.y & 0xFFu);
+            auto place = [&](const TailChild &c, long long rank) {
+                const int ks = (int)(c.pk & 0xFFu), sg = (int)((c.pk >> 8) & 1u);
                 if (rank >= room) {
                     ++ty.spawn_drop;
                     ty.q_drop += (uint32_t)ks;
                     return;
                 }
-                int layer = (int)((rec.y >> 8) & 0xFu);
-                const uint32_t g0 = (rec.y >> 12) & 0xFFu, gen = g0 < 255u ? g0 + 1u : 255u;
-                const uint4 y = philox_rk(make_uint4((uint32_t)pslot, x.ctr_hi, step, SUB_SEC), a);
-                const int sg = y.x < s_p0[layer] ? 0 : 1;
-                const float zb = __uint_as_float(rec.x);
-                float z = zb, mu = mu_of(y.y), lo = s_edge[layer], hi = s_edge[layer + 1];
-                TabEnt e = s_ent[(layer * 2 + sg) * x.ne + (ks - 1)];
-                flight<DET>(a, S, z, mu, layer, e, lo, hi, sg, ks, half, (uint32_t)pslot, x.ctr_hi, step,
-                            SUB_SIF, ty);
+                ty.hits += c.hits;
+                ty.trans += c.trans;
+                ty.trunc += c.trunc;
                 const unsigned long long id = nid + (unsigned long long)rank;
                 const long long d = nsl + rank;
-                x.Z[d] = z;
+                x.Z[d] = c.z;
                 *reinterpret_cast<uint2 *>(x.MU + 2 * d) =
-                    make_uint2(__float_as_uint(mu), (uint32_t)ks | ((uint32_t)sg << 8) | ((uint32_t)layer << 9) |
-                                                        (gen << 13) | ((uint32_t)(id >> 32) << 21));
+                    make_uint2(__float_as_uint(c.mu), c.pk | ((uint32_t)(id >> 32) << 21));
                 x.ID[d] = (uint32_t)id;
                 ++kept_here;
                 uint32_t wp = 0;
                 if (a.w[0]) {
-                    wp = __ldcg(&x.W[pslot]);
+                    wp = __ldcg(&x.W[c.pslot]);
                     x.W[d] = wp;
                 }
-                tail_birth(a, x, t, sg, zb, wp);
-                if (dep) tail_deposit(a, x, t, sg, ks, gen, z, __fmul_rn(e.v, mu));
+                tail_birth(a, x, t, sg, c.zb, wp);
+                if (dep) tail_deposit(a, x, t, sg, ks, (c.pk >> 13) & 0xFFu, c.z, __fmul_rn(c.v, c.mu));
             };
             if (s_tot[j] > 0) {
-                // pieces of the block's sub-tiles: a prefix of their counts,
-                // then a thread per record
+                // a thread per record, in pieces of the block's sub-tiles
                 long long run = s_mine[j];
-                for (long long p0 = u0; p0 < u1; p0 += TAIL_PIECE) {
-                    const int np = (int)(u1 - p0 < TAIL_PIECE ? u1 - p0 : TAIL_PIECE);
-                    int c[TAIL_PIECE / TPB], sum = 0;
-#pragma unroll
-                    for (int q = 0; q < TAIL_PIECE / TPB; ++q) {
-                        const int i = tid * (TAIL_PIECE / TPB) + q;
-                        c[q] = i < np ? (int)cnt[j * g.cnt_n + p0 + i] : 0;
-                        sum += c[q];
-                    }
-                    int excl;
-                    const int tot = block_scan(sum, excl, s_w);
-                    if (tot == 0) continue;
-#pragma unroll
-                    for (int q = 0; q < TAIL_PIECE / TPB; ++q) {
-                        s_pre[tid * (TAIL_PIECE / TPB) + q] = (uint32_t)excl;
-                        excl += c[q];
-                    }
-                    if (tid == 0) s_pre[TAIL_PIECE] = (uint32_t)tot;
-                    cta_sync();
+                if (tid < tot0) place(ch, run + tid);
 #pragma unroll 1
-                    for (int r = tid; r < tot; r += TPB) {
-                        int lo = 0, hi = TAIL_PIECE - 1;         // last sub-tile with prefix <= r
-                        while (lo < hi) {
-                            const int mid = (lo + hi + 1) >> 1;
-                            if (s_pre[mid] <= (uint32_t)r) lo = mid; else hi = mid - 1;
-                        }
-                        const long long sl0 = (p0 + lo) * g.sub;
-                        const uint2 rec = __ldcg(&list[sl0 + (r - (int)s_pre[lo])]);
-                        place(rec, sl0 + (rec.y >> 20), run + r);
-                    }
-                    run += tot;
+                for (int r = tid + TPB; r < tot0; r += TPB) place(record(j, u0, r), run + r);
+                run += tot0;
+                for (long long p0 = u0 + TAIL_PIECE; p0 < u1; p0 += TAIL_PIECE) {
                     cta_sync();
+                    const int tot = prefix(j, p0, (int)(u1 - p0 < TAIL_PIECE ? u1 - p0 : TAIL_PIECE));
+#pragma unroll 1
+                    for (int r = tid; r < tot; r += TPB) place(record(j, p0, r), run + r);
+                    run += tot;
                 }
             }
             if (tail_tot > 0) {
@@ -1127,7 +1189,7 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
                     const uint2 rec = p0 + tid < x1 ? list[slot] : make_uint2(0u, 0u);
                     int excl;
                     const int tot = block_scan((rec.y & 0xFFu) != 0u ? 1 : 0, excl, s_w);
-                    if ((rec.y & 0xFFu) != 0u) place(rec, slot, run + excl);
+                    if ((rec.y & 0xFFu) != 0u) place(make(step, rec, slot), run + excl);
                     run += tot;
                 }
             }
@@ -1152,7 +1214,11 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
             nid += (unsigned long long)i1;
             adds += (unsigned long long)(i0 + kept + i1);
             // the carriers written here are read by other blocks in the next step
-            if (j + 1 < sp.len && nsl > n0) stack_sync(a, bar, bar_t += (unsigned int)nbk);
+            if (j + 1 < sp.len) {
+                if (nsl > n0) stack_arrive(bar); else cta_sync();
+                prepare(j + 1);
+                if (nsl > n0) stack_wait(a, bar, bar_t += (unsigned int)nbk);
+            }
         }
         // ---- the block's counts
         const uint32_t vals[10] = {ty.absorbed, ty.bath, ty.hits, ty.trans, ty.trunc, ty.spawn_drop,
