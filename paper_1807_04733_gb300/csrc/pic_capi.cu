@@ -802,8 +802,11 @@ pic_status pic_init(pic_ctx **out, const pic_params *p, const pic_stack_desc *st
     a.qcnt = c->d_qcnt;
     a.fspawn = c->d_fspawn;
 
-    // grouped steps, where their shared memory fits
-    e = configure_group(a, c->total_slots, &c->gc);
+    // grouped steps, where their shared memory fits and no threshold is within
+    // 2^-16 of one (their first test rounds thresholds up)
+    bool rounds = true;
+    for (const TabEnt &x : ent) rounds = rounds && x.P < 0xFFFF0000u;
+    if (rounds) e = configure_group(a, c->total_slots, &c->gc);
     std::vector<int4> blk;
     if (e == cudaSuccess && c->gc.ok) {
         GroupArgs &g = c->ga;

@@ -137,11 +137,12 @@ __device__ __forceinline__ uint2 *list_of(const GroupArgs &g, int j)
     return p + (j & 1) * g.list_n;
 }
 
-// A slot's test word: the upper half of its threshold, and the edge ahead as
-// a half-precision number rounded down (its sign kept, that of zero too).
+// A slot's test word: the upper half of its threshold plus one, and the edge
+// ahead as a half-precision number rounded down (its sign kept, that of zero
+// too).  A random word below the threshold is below the test word.
 __device__ __forceinline__ uint32_t test_word(uint32_t P, float edge)
 {
-    return (P & 0xFFFF0000u) | (uint32_t)__half_as_ushort(__float2half_rd(edge));
+    return (P ? (P & 0xFFFF0000u) + 0x10000u : 0u) | (uint32_t)__half_as_ushort(__float2half_rd(edge));
 }
 
 __device__ __forceinline__ float edge_of(uint32_t t)
@@ -150,7 +151,7 @@ __device__ __forceinline__ float edge_of(uint32_t t)
 }
 
 struct GroupSmem {               // byte offsets in dynamic shared memory
-    size_t ent, mv, base, q, t, j, n, gs, v, tiles, warps, total, per_warp;
+    size_t ent, mv, q, t, j, n, gs, v, tiles, warps, total, per_warp;
 };
 
 // Shared memory of a warp: per slot the depth, the speed, the test word (upper
@@ -169,8 +170,7 @@ __host__ __device__ inline GroupSmem group_smem(const Args &a, bool dep, int qua
     auto up = [](size_t x) { return (x + 15) & ~(size_t)15; };
     size_t p = 0;
     o.ent = p; p = up(p + (size_t)a.ftab_max * sizeof(FastEnt));
-    o.mv = p; p = up(p + (size_t)a.ftab_max * 8);
-    o.base = p; if (dep) p = up(p + (size_t)a.ftab_max * 4);
+    o.mv = p; p = up(p + (size_t)a.ftab_max * 16);
     o.q = p; p = up(p + (size_t)a.tab_max * 4);
     o.t = p; p = up(p + (size_t)a.T_max * 4);
     o.j = p; p = up(p + (size_t)nj * a.jbin_max * 4);
@@ -227,8 +227,7 @@ __device__ __forceinline__ void phase_group(const Args &a, const GroupArgs &g, c
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NT = (int)blockDim.x;
     const GroupSmem o = group_smem(a, DEP, Q, 0, g.nd, g.nj);
     FastEnt *s_ent = reinterpret_cast<FastEnt *>(smem + o.ent);
-    uint32_t *s_mv = reinterpret_cast<uint32_t *>(smem + o.mv);      // test words by 2 * index + down
-    uint32_t *s_bw = reinterpret_cast<uint32_t *>(smem + o.base);    // bin words by index
+    uint4 *s_mv = reinterpret_cast<uint4 *>(smem + o.mv);    // speed, test words up and down, bin row
     uint32_t *s_Q = reinterpret_cast<uint32_t *>(smem + o.q);
     uint32_t *s_T = reinterpret_cast<uint32_t *>(smem + o.t);
     int32_t *s_J = reinterpret_cast<int32_t *>(smem + o.j);
@@ -284,14 +283,11 @@ __device__ __forceinline__ void phase_group(const Args &a, const GroupArgs &g, c
         for (int i = tid; i < st.ftab_n; i += NT) {
             const FastEnt e = a.fent[st.fent_off + i];
             s_ent[i] = e;
-            s_mv[2 * i] = test_word(e.P, e.hi);
-            s_mv[2 * i + 1] = test_word(e.P, -e.lo);
-            if (DEP) {
-                // byte offset of the (spin, k) row of bins; removed slots have a
-                // row of their own after the last
-                const int k = i & ((1 << a.kb) - 1), sg = (i >> a.kb) & 1;
-                s_bw[i] = (uint32_t)(4 * (k >= 1 && k <= ne ? (sg * ne + k - 1) * nc : nb));
-            }
+            // byte offset of the (spin, k) row of bins; removed slots have a row
+            // of their own after the last
+            const int k = i & ((1 << a.kb) - 1), sg = (i >> a.kb) & 1;
+            s_mv[i] = make_uint4(__float_as_uint(e.v), test_word(e.P, e.hi), test_word(e.P, -e.lo),
+                                 (uint32_t)(4 * (k >= 1 && k <= ne ? (sg * ne + k - 1) * nc : nb)));
         }
         for (int i = tid; i < st.tab_n; i += NT) s_Q[i] = a.ent[st.ent_off + i].Q;
         for (int i = tid; i < st.T_n; i += NT) s_T[i] = a.T_thr[st.T_off + i];
@@ -318,6 +314,7 @@ __device__ __forceinline__ void phase_group(const Args &a, const GroupArgs &g, c
             const int sub = (int)(ta - s_tpref[s]) + (int)u;     // sub-tile of the stack
             const int slot0 = sub * S;
             const int nvalid = nsl - slot0;                      // at least 1
+            const bool ragged = nvalid < S;
             // ---- load: quads of consecutive lanes are consecutive in memory
 #pragma unroll
             for (int q = 0; q < Q; ++q) {
@@ -332,14 +329,14 @@ __device__ __forceinline__ void phase_group(const Args &a, const GroupArgs &g, c
                 uint32_t to[4], bo[4];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
-                    const uint32_t pk = i4 + c < nvalid ? pi[c] : 0u;
-                    const int idx = fast_index(a, pk);
-                    const float w = __fmul_rn(s_ent[idx].v, __uint_as_float(mi[c]));
+                    const uint32_t pk = ragged && i4 + c >= nvalid ? 0u : pi[c];
+                    const uint4 e = s_mv[fast_index(a, pk)];
+                    const float w = __fmul_rn(__uint_as_float(e.x), __uint_as_float(mi[c]));
                     const bool dn = w < 0.f;
                     zo[c] = dn ? -zi[c] : zi[c];
                     wo[c] = dn ? -w : w;
-                    to[c] = s_mv[2 * idx + (dn ? 1 : 0)];
-                    if (DEP) bo[c] = s_bw[idx] | ((pk & 0xFFu) ? ((pk >> 13) & 0xFFu) << 24 : 0u);
+                    to[c] = dn ? e.z : e.y;
+                    if (DEP) bo[c] = e.w | ((pk & 0xFFu) ? (pk << 11) & 0xFF000000u : 0u);
                 }
                 const int i = q * 32 + lane, v = (i / Q) * RQ + i % Q;
                 wz[v] = make_float4(zo[0], zo[1], zo[2], zo[3]);
@@ -385,7 +382,7 @@ __device__ __forceinline__ void phase_group(const Args &a, const GroupArgs &g, c
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
                             const float z2 = fly<DET>(fly<DET>(zi[c], wi[c], half), wi[c], half);
-                            const bool slow = (z2 > edge_of(ti[c])) | (xi[c] < (ti[c] | 0xFFFFu));
+                            const bool slow = (z2 > edge_of(ti[c])) | (xi[c] < ti[c]);
                             zo[c] = slow ? zi[c] : z2;
                             if (slow) nib |= 1u << c;
                             if (D) {
@@ -595,13 +592,13 @@ __device__ __forceinline__ void phase_group(const Args &a, const GroupArgs &g, c
                         }
                         const float w = __fmul_rn(e.v, mu);
                         const bool dn = w < 0.f;
-                        const int idx = fast_index(a, pk);
+                        const uint4 en = s_mv[fast_index(a, pk)];
                         reinterpret_cast<float *>(wz)[pv] = dn ? -z : z;
                         reinterpret_cast<float *>(ww)[pv] = dn ? -w : w;
-                        reinterpret_cast<uint32_t *>(wt)[pv] = s_mv[2 * idx + (dn ? 1 : 0)];
+                        reinterpret_cast<uint32_t *>(wt)[pv] = dn ? en.z : en.y;
                         if (DEP) {
                             reinterpret_cast<uint32_t *>(wb)[pv] =
-                                s_bw[idx] | ((pk & 0xFFu) ? ((pk >> 13) & 0xFFu) << 24 : 0u);
+                                en.w | ((pk & 0xFFu) ? (pk << 11) & 0xFF000000u : 0u);
                             if (dep && (pk & 0xFFu)) {
                                 const int ce = cell_at(z, a.inv_dz, nc);
                                 atomicAdd(&h_n[(sg * ne + k - 1) * nc + ce], 1u);
