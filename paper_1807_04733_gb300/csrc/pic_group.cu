@@ -1276,7 +1276,8 @@ __global__ void __launch_bounds__(TPB, 2) k_tail(const Args a, const GroupArgs g
 // step before ended, from the state: 12 bytes read per slot and two or three
 // shared-memory additions per carrier.
 // ---------------------------------------------------------------------------
-constexpr int DENS_T = 512;
+constexpr int DENS_T = 1024;     // (with 512 threads and branches around the additions 1.06 ms
+                                 // for 4e8 slots, now 0.72: the bandwidth of a copy)
 
 __device__ __forceinline__ void phase_dens(const Args &a)
 {
@@ -1323,6 +1324,7 @@ __device__ __forceinline__ void phase_dens(const Args &a)
             for (int i = tid; i < st.ftab_n; i += NT) s_ent[i] = a.fent[st.fent_off + i];
         }
         __syncthreads();
+        const uint32_t a_n = smem_addr(s_n), a_gs = smem_addr(s_gs);
         const float *Z = a.z[cur] + st.base;
         const float *MU = a.mu[cur] + 2 * st.base;
         const long long i0 = (ta - s_tpref[s]) * TILE;
@@ -1337,13 +1339,15 @@ __device__ __forceinline__ void phase_dens(const Args &a)
             const uint32_t pi[4] = {m0.y, m0.w, m1.y, m1.w}, mi[4] = {m0.x, m0.z, m1.x, m1.z};
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                const uint32_t pk = pi[c];
+                // a removed slot adds 0 to the first row (z of a slot past the last
+                // one may be anything: its cell is held inside)
+                const uint32_t pk = i + c < i1 ? pi[c] : 0u;
                 const int k = (int)(pk & 0xFFu), sg = (int)((pk >> 8) & 1u);
-                if (k == 0 || i + c >= i1) continue;
-                const int cl = cell_at(zi[c], a.inv_dz, nc);
-                atomicAdd(&s_n[(sg * ne + k - 1) * nc + cl], 1u);
-                atomicAdd(&s_gs[cl], (pk >> 13) & 0xFFu);
-                if (vmom)
+                const uint32_t on = k != 0 ? 1u : 0u;
+                const int cl = max(cell_at(zi[c], a.inv_dz, nc), 0);
+                red_shared(a_n + 4u * (uint32_t)((on ? sg * ne + k - 1 : 0) * nc + cl), on);
+                red_shared(a_gs + 4u * (uint32_t)cl, on ? (pk >> 13) & 0xFFu : 0u);
+                if (vmom && on)
                     add_u64_split(&s_v[sg * nc + cl],
                                   (unsigned long long)vel_q(__fmul_rn(s_ent[fast_index(a, pk)].v,
                                                                       __uint_as_float(mi[c]))));
