@@ -1293,10 +1293,25 @@ __device__ __forceinline__ void phase_stream(const Args &a)
                     if (i0 + j < nvalid) gA[j] = av[j];
             }
         }
-        // queue the eventful carriers (record and position), in tile order:
-        // the warp's exclusive prefix of the per-thread counts (0..G) from
-        // ballots of their bits, one shared-counter reservation per warp
-        {
+        // queue the eventful carriers (record and position).  Only the stacks'
+        // order matters to k_event (the barriers at a stack's end keep it), so a
+        // lane that has some reserves its entries by itself: a prefix over the
+        // warp took four times the instructions of this.
+        if constexpr (!EV) {
+            if (slowbits) {
+                const int cnt = __popc(slowbits);
+                n_queued += (uint32_t)cnt;
+                float4 *dst = a.qrec + pos0 + atomicAdd(&s_qn, cnt);
+                const uint32_t rel = (uint32_t)((t - t0) * TILE) + (uint32_t)i0;
+#pragma unroll
+                for (int j = 0; j < G; ++j)
+                    if ((slowbits >> j) & 1u)
+                        *dst++ = make_float4(zin[j], min_[j], __uint_as_float(pin[j]),
+                                             __uint_as_float(rel + (uint32_t)j));
+            }
+        } else {
+            // the event ring: positions from the warp's exclusive prefix of the
+            // per-thread counts (0..G) by ballots of their bits
             const uint32_t cnt = (uint32_t)__popc(slowbits);
             constexpr int NB = G == 4 ? 3 : 4;       // bits of a count 0..G
             unsigned int bal[NB];
@@ -1306,7 +1321,7 @@ __device__ __forceinline__ void phase_stream(const Args &a)
                 bal[q] = __ballot_sync(0xffffffffu, (cnt >> q) & 1u);
                 tot += __popc(bal[q]) << q;
             }
-            if (tot && EV) {
+            if (tot) {
                 // fused form: into the event ring, after the depths above
                 unsigned int base = 0;
                 if (lane == 0) base = atomicAdd(&s_etail, (unsigned int)tot);
@@ -1339,22 +1354,6 @@ __device__ __forceinline__ void phase_stream(const Args &a)
                     __threadfence_block();       // the record and this tile's depths first
                     *sq = 2u * p + 1u;
                     ++p;
-                }
-            } else if (tot) {
-                int base = 0;
-                if (lane == 0) base = atomicAdd(&s_qn, tot);
-                base = __shfl_sync(0xffffffffu, base, 0);
-                long long q = pos0 + base;
-#pragma unroll
-                for (int r = 0; r < NB; ++r) q += (long long)(__popc(bal[r] & lt_mask) << r);
-                n_queued += cnt;
-                const uint32_t rel = (uint32_t)((t - t0) * TILE) + (uint32_t)i0;
-#pragma unroll
-                for (int j = 0; j < G; ++j) {
-                    if ((slowbits >> j) & 1u) {
-                        a.qrec[q++] = make_float4(zin[j], min_[j], __uint_as_float(pin[j]),
-                                                  __uint_as_float(rel + (uint32_t)j));
-                    }
                 }
             }
         }
