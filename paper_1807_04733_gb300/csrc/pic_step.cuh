@@ -1641,6 +1641,8 @@ __device__ __forceinline__ void phase_place(const Args &a)
     __shared__ unsigned long long s_r8[(TPB / 32) * 8];    // block sums of the ledger counts
     __shared__ long long s_pre[2], s_cl;
     __shared__ int s_flag;
+    constexpr int PLACE_LIST = 2048;             // positions (of at most 8 TPB words) held at a time
+    __shared__ uint16_t s_list[PLACE_LIST];
 
     const unsigned int ep = *(volatile unsigned int *)&a.ctl->epoch;
     const int cur = (int)*(volatile unsigned int *)&a.ctl->cur;
@@ -1763,18 +1765,26 @@ __device__ __forceinline__ void phase_place(const Args &a)
                 for (int u = 0; u < PW; ++u)
                     if (wd[u]) a.spawn_bits[wt + u] = 0u;
             }
-            long long g = run + excl;
+            // the positions in order into shared memory, then a thread per
+            // secondary (a thread that walked its own bits did them one after
+            // another)
 #pragma unroll 1
-            for (int u = 0; u < q; ++u) {
-                uint32_t bits = wd[0];                  // word u, by selects (no local array)
+            for (int b0 = 0; b0 < tot; b0 += PLACE_LIST) {
+                int o = excl - b0;
+                if (cnt && o < PLACE_LIST && o + cnt > 0) {
 #pragma unroll
-                for (int v = 1; v < PW; ++v)
-                    if (u == v) bits = wd[v];
-                const long long w = wt + u;
-                while (bits) {
-                    const int j = __ffs(bits) - 1;
-                    bits &= bits - 1u;
-                    const float4 r = a.stage[w * 32 + j];
+                    for (int u = 0; u < PW; ++u)
+                        for (uint32_t bits = wd[u]; bits; bits &= bits - 1u, ++o)
+                            if (o >= 0 && o < PLACE_LIST)
+                                s_list[o] = (uint16_t)((q * tid + u) * 32 + __ffs(bits) - 1);
+                }
+                cta_sync();
+                const int here = tot - b0 < PLACE_LIST ? tot - b0 : PLACE_LIST;
+#pragma unroll 1
+                for (int v = tid; v < here; v += TPB) {
+                    const long long pos = wb * 32 + (long long)s_list[v];
+                    const long long g = run + b0 + v;
+                    const float4 r = a.stage[pos];
                     const uint32_t pk_staged = __float_as_uint(r.z);
                     const uint32_t pk = pk_staged & 0x1FFFFFu;
                     if (g < room) {
@@ -1791,13 +1801,12 @@ __device__ __forceinline__ void phase_place(const Args &a)
                         const int sg = (int)((pk >> 8) & 1u), k = (int)(pk & 0xFFu);
                         const int c0 = cell_of(a, tmp, r.w), c1 = cell_of(a, tmp, r.x);
                         if (ADJ) {
-                            place_adj(s, stg, w * 32 + j, d, id, pk, sg, k, c0, c1, r);
+                            place_adj(s, stg, pos, d, id, pk, sg, k, c0, c1, r);
                         } else {
                             // a birth, where the parent created it; the
                             // secondary carries its parent's weight
                             atomicAdd(&s_J[sg * nf + c0], 1);
                             if (a.w[0]) {
-                                const long long pos = w * 32 + j;
                                 const uint32_t wp = a.w[cur][stg.base + pos - s_tpref[s] * TILE];
                                 a.w[cur][d] = wp;
                                 atomicAdd(reinterpret_cast<unsigned long long *>(a.bdw) + stg.J_off +
@@ -1819,8 +1828,8 @@ __device__ __forceinline__ void phase_place(const Args &a)
                         ++ty.spawn_drop;
                         ty.q_drop += pk & 0xFFu;
                     }
-                    ++g;
                 }
+                cta_sync();
             }
             run += tot;
             wb += span;
