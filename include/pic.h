@@ -98,7 +98,10 @@ typedef struct {
                                cooperative launch (every block resident, the
                                passes of every step separated by grid barriers
                                with bounded waits), captured in a CUDA graph;
-                               0: one launch per kernel.  Results are
+                               grouped steps (event_pass 0) run each call of
+                               pic_step in one such launch; 0: one launch per
+                               kernel, or for grouped steps of up to 2^23 slots
+                               the single launch of 2.  Results are
                                identical; kernel timing (pic_profile) always
                                uses single launches. */
     int32_t stack_base;     /* global index of the context's first stack
@@ -111,13 +114,18 @@ typedef struct {
                                carriers, 4 or 8 (each thread then takes 8 or 4
                                consecutive slots of a 1024-slot tile); 0 = 8.
                                Results do not depend on it. */
-    int32_t event_pass;     /* 0: the ordinary steps of a single-stack context
-                               with eight consumer warps run the general step
-                               of the eventful carriers inside the streaming
-                               pass (extra warps fed through a shared-memory
-                               ring, while the carriers' sectors are in L2);
-                               1: always a separate event pass after the
-                               streaming pass.  Results do not depend on it. */
+    int32_t event_pass;     /* 0: the steps run in groups, several per pass over
+                               memory; where that does not fit (a moment grid
+                               of more than the shared memory, scattering
+                               probabilities within 2^-16 of 1), the ordinary
+                               steps of a single-stack context with eight
+                               consumer warps run the general step of the
+                               eventful carriers inside the streaming pass
+                               (extra warps fed through a shared-memory ring,
+                               while the carriers' sectors are in L2);
+                               1: single steps, each with a separate event
+                               pass after the streaming pass.  Results do not
+                               depend on it. */
 } pic_params;
 
 /* Launch configuration a context chose (pic_launch_info). */
@@ -204,6 +212,9 @@ typedef struct {
 /* Device time of the library's kernels, per kind: 0 = source, 1 = step
  * (streaming pass), 2 = step with density deposit (streaming pass),
  * 3 = compaction, 4 = step (event pass and placement of secondaries);
+ * grouped steps (several per launch): 1 or 2 = the pass over the carriers,
+ * without or with density deposit, 2 also the separate density pass, 4 = new
+ * carriers and their steps;
  * pic_grad's replays: 5 = streaming pass, 6 = event pass, 7 = the rest
  * (source, compaction, flux potential, flush, lineage totals);
  * 8 = the fluxes derived by pic_moments and pic_weighted_moments;
@@ -435,15 +446,16 @@ typedef struct {
 
 /* Time candidate launch configurations of the step kernels on the running
  * simulation and keep the fastest.  Each candidate advances every stack by
- * trial_steps ordinary steps (results do not depend on the launch
- * configuration: the slot order and every random word are fixed by the
- * run), timed with CUDA events on the context stream and divided by the
- * carriers advanced.  Candidates: 8 or 4 consumer warps per block of the
- * streaming pass (4 or 8 slots per thread), 1 to 6 (8 with four warps)
- * resident blocks per SM, ring depth 2, 3, 4, 6 or 8 where it fits, both
- * deposit modes when the trial contains density steps, and (eight consumer
- * warps, a single stack) the general step inside the streaming pass or in a
- * separate pass.  entries (host, may be NULL): up to max_entries results in
+ * trial_steps ordinary steps, grouped ones (event_pass 0) by at least a whole
+ * group (results do not depend on the launch configuration: the slot order
+ * and every random word are fixed by the run), timed with CUDA events on the
+ * context stream and divided by the carriers advanced.  Candidates: grouped
+ * steps, where the context can run them; single steps with 8 or 4 consumer
+ * warps per block of the streaming pass (4 or 8 slots per thread), 1 to 6 (8
+ * with four warps) resident blocks per SM, ring depth 2, 3, 4, 6 or 8 where
+ * it fits, both deposit modes when the trial contains density steps; and,
+ * where steps cannot be grouped (eight consumer warps, a single stack), the
+ * general step inside the streaming pass or in a separate pass.  entries (host, may be NULL): up to max_entries results in
  * the order tried; *n_entries (may be NULL): their number.  Needs steps left:
  * up to 200 * trial_steps.  Synchronises. */
 pic_status pic_autotune(pic_ctx *ctx, int trial_steps, pic_tune_entry *entries,

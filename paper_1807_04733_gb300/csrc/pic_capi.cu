@@ -2135,8 +2135,14 @@ pic_status pic_autotune(pic_ctx *c, int trial_steps, pic_tune_entry *entries, in
                         if (ev == 0 && grp && (ring != 2 || hm != 0)) continue;
                         cands.push_back({bps, ring, hm, nw, ev});
                     }
-    if ((int64_t)c->step + (int64_t)trial_steps * (int64_t)cands.size() > c->p.n_steps_max)
+    // a trial of grouped steps has at least a whole group (with two steps where a
+    // group has four the spin valve's were taken for slower than single ones);
+    // the budget of steps is that of single ones, one trial per configuration
+    auto steps_of = [&](const Cand &k) { return k.ev == 0 && grp ? std::max(trial_steps, c->gc.m) : trial_steps; };
+    const int64_t budget = (int64_t)trial_steps * (dep_in_trial ? 2 : 1) * 5 * ((fusable ? 3 : 0) + 6 + 8);
+    if ((int64_t)c->step + budget > c->p.n_steps_max)
         return fail(c, PIC_ERR_ARG, "pic_autotune: not enough steps left for the trials");
+    const int32_t first_step = c->step;
     const int use_graph = c->p.use_graph;
     c->p.use_graph = 0;                       // trials use single launches
     cudaEvent_t ev[2] = {nullptr, nullptr};
@@ -2163,6 +2169,7 @@ pic_status pic_autotune(pic_ctx *c, int trial_steps, pic_tune_entry *entries, in
     std::vector<pic_tune_entry> res;
     for (size_t i = 0; i < cands.size() && e == cudaSuccess; ++i) {
         const Cand &k = cands[i];
+        if ((int64_t)(c->step - first_step) + steps_of(k) > budget) continue;
         LaunchCfg lc{};
         if (configure(c->args, k.bps, k.ring, k.hm, k.nw, &lc) != cudaSuccess) {
             cudaGetLastError();               // does not fit: not a candidate
@@ -2185,7 +2192,7 @@ pic_status pic_autotune(pic_ctx *c, int trial_steps, pic_tune_entry *entries, in
         e = steps_done(ps0);
         if (e == cudaSuccess) e = cudaEventRecord(ev[0], c->stream);
         if (e != cudaSuccess) break;
-        const pic_status st = pic_step(c, trial_steps);
+        const pic_status st = pic_step(c, steps_of(k));
         if (st != PIC_OK) {
             c->lc = keep;
             c->p = keep_p;
