@@ -36,14 +36,11 @@ namespace pic {
 
 namespace {
 
-#ifndef PIC_GROUP_UNROLL
-#define PIC_GROUP_UNROLL 4
-#endif
-#ifndef PIC_GROUP_GW
-#define PIC_GROUP_GW 16
-#endif
-constexpr int GW_MAX = PIC_GROUP_GW;       // most warps of a k_group block
-constexpr int UNROLL = PIC_GROUP_UNROLL;
+// Most warps of a k_group block (20 and 24, at the fewer registers that leaves,
+// were not faster) and quads per turn of the sweep (2: 39.9 ms for 50 steps of
+// 4e8 carriers, 4: 39.5).
+constexpr int GW_MAX = 16;
+constexpr int UNROLL = 4;
 
 template <bool DET>
 __device__ __forceinline__ float fly(float z, float w, float t)
@@ -1461,9 +1458,6 @@ cudaError_t configure_group(const Args &a, long long slots, GroupCfg *gc)
     c.quads = c.dep ? 4 : 8;
     if (slots < (long long)sms * 12 * 1024) c.quads = 4;
     if (slots < (long long)sms * 12 * 512) c.quads = 2;
-#ifdef PIC_GROUP_Q
-    if (c.quads > PIC_GROUP_Q) c.quads = PIC_GROUP_Q;
-#endif
     for (int m = slots <= GROUP_LIST_SLOTS ? GROUP_OPEN : GROUP_OPEN_LARGE; m >= 1 && !c.ok; --m) {
         const int nd = c.dep ? (me - 1 + m) / me : 0;
         const int nj = c.dep ? (me + m - 2) / me + 1 : 1;

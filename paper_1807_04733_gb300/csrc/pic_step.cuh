@@ -1,8 +1,10 @@
 // Device code of the PIC step (sm_103a): helpers and the kernel templates.
-// Included by pic_kernels.cu (the forward step) and pic_adjoint.cu (the
-// adjoint replay); each translation unit instantiates what it launches.
+// Included by pic_kernels.cu (single forward steps, source, compaction),
+// pic_adjoint.cu (the adjoint replay) and pic_group.cu (forward steps in
+// groups, the default, which shares the helpers and the general step); each
+// translation unit instantiates what it launches.
 //
-// One Strang step (Eq. strang, Sec. III.A) is, per stack:
+// One Strang step (Eq. strang, Sec. III.A), run by itself, is, per stack:
 //   k_inject(half 0)   Source(dt/2): append new carriers
 //   k_stream           Transport(dt/2) -> Scattering(dt) -> Transport(dt/2)
 //                      for every carrier that neither scatters nor meets a
@@ -353,12 +355,6 @@ static __device__ long long look_back_warp(const Args &a, unsigned int ep, long 
         if (term) break;
     }
     return prefix;
-}
-
-__device__ __forceinline__ long long look_back(const Args &a, unsigned int ep, long long T,
-                                               long long ts, int b, int G)
-{
-    return look_back_warp(a, ep, ts, b, [&](int j) { return T * j / G; });
 }
 
 // Per-block plan shared by the streaming kernels: tiles of every stack
