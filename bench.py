@@ -68,8 +68,9 @@ def parse():
                     help="1: the main line replays whole periods from CUDA graphs (use_graph); "
                          "0: one launch per kernel")
     ap.add_argument("--event-pass", type=int, default=0, choices=(0, 1),
-                    help="ordinary steps: 0 general step inside the streaming pass where it "
-                         "applies, 1 separate event pass (the autotuner may change it)")
+                    help="0 grouped steps (or the general step inside the streaming pass where "
+                         "they do not apply), 1 single steps with a separate event pass (the "
+                         "autotuner may change it)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--cpu-seconds", type=float, default=15.0)
     ap.add_argument("--no-adjoint", action="store_true")
@@ -132,9 +133,36 @@ def measured_peak():
 NCU_TRAFFIC = {"separate": 16.76, "fused": 14.81, "src_sha": "59659cabec44282e"}
 
 
-def kernel_sha():
-    with open(os.path.join(ROOT, "paper_1807_04733_gb300", "csrc", "pic_step.cuh"), "rb") as f:
+def kernel_sha(name="pic_step.cuh"):
+    with open(os.path.join(ROOT, "paper_1807_04733_gb300", "csrc", name), "rb") as f:
         return hashlib.sha256(f.read()).hexdigest()[:16]
+
+
+# Grouped steps hold a carrier in shared memory through many time steps, so
+# memory is not what bounds them: instruction issue is.  Warp instructions that a
+# carrier-step needs: a quarter of a Philox4x32-10 call and the two half flights
+# with their three comparisons for every carrier (14 per lane), about 250 per 32
+# eventful ones; issue slots per second from the SM count and the clock.
+WARP_INST_STEP, WARP_INST_EVENT = 14.0 / 32.0, 250.0 / 32.0
+# DRAM bytes per carrier-step of k_group's closed groups (the large bilayer scaled
+# to 1/20, 46 steps in a pass), valid for the source whose hash is given
+NCU_GROUP = {"bytes": 0.458, "src_sha": "2c885175345e7be5"}
+
+
+def grouped_roofline(delta, k_ms, ms, time_steps, sms=152, sm_ghz=2.07):
+    ps = delta["particle_steps"]
+    need = (WARP_INST_STEP * ps + WARP_INST_EVENT * delta["eventful"]) / ps if ps else WARP_INST_STEP
+    peak = sms * 4 * sm_ghz * 1e9 / need
+    achieved = ps / (k_ms * 1e-3)
+    pinned = NCU_GROUP["bytes"] is not None and NCU_GROUP["src_sha"] == kernel_sha("pic_group.cu")
+    return {"bound": "issue", "achieved": achieved, "peak": peak, "unit": "particle-steps/s",
+            "frac": achieved / peak, "form": "grouped",
+            "kernel": "k_group + k_tail (several time steps per pass over memory), k_dens",
+            "peak_source": "%d SMs x 4 issue slots x %.2f GHz / %.2f warp instructions needed per "
+                           "carrier-step" % (sms, sm_ghz, need),
+            "traffic": NCU_GROUP["bytes"] * ps / time_steps if pinned else None,
+            "avg_launch_ms": k_ms / time_steps,
+            "kernel_share_of_step_time": k_ms / ms if ms else 0}
 
 
 class Clocks:
@@ -463,8 +491,9 @@ def batched_leg(args):
 # ---------------------------------------------------------------------------
 # roofline of the step kernels and timed legs of other configurations
 # ---------------------------------------------------------------------------
-def roofline_of(delta, ktimes, ms, fused=False):
-    """The step kernels: the streaming pass (k_stream), the event pass
+def roofline_of(delta, ktimes, ms, fused=False, time_steps=None):
+    """`time_steps` steps in fewer launches: grouped steps (grouped_roofline).
+    Else the step kernels: the streaming pass (k_stream), the event pass
     (k_event) and the placement of secondaries (k_place), or, fused (the
     ordinary steps of a context whose launch configuration has the general
     step inside the streaming pass), k_stream and k_place; one launch of each
@@ -475,6 +504,8 @@ def roofline_of(delta, ktimes, ms, fused=False):
     k_ms = ktimes["step"][1] + ktimes["step_moments"][1] + ktimes["step_events"][1]
     if not n_k or not k_ms:
         return None
+    if time_steps and n_k < time_steps:
+        return grouped_roofline(delta, k_ms, ms, time_steps)
     alg = B_STEP * delta["particle_steps"] + B_EVENTFUL * delta["eventful"] + \
         B_CHANGED * delta["changed"] + B_SPAWN * delta["spawned"]
     strict = S_STEP * delta["particle_steps"] + S_EVENTFUL * delta["eventful"] + \
@@ -546,7 +577,8 @@ def timed_leg(wl, pre, n_timed, chunk, capacity=None, autotune_steps=0):
     lcfg = ctx.launch_config()
     out = {"value": delta["particle_steps"] / (ms * 1e-3), "unit": UNIT, "ms": ms,
            "time_steps": n_timed,
-           "roofline": roofline_of(delta, kt, ms, fused=lcfg["grid_step_fused"] > 0),
+           "roofline": roofline_of(delta, kt, ms, fused=lcfg["grid_step_fused"] > 0,
+                                   time_steps=n_timed),
            "saturation": saturation(delta), "ledger_delta": delta,
            "kernel_ms": {k: v[1] for k, v in kt.items() if v[0]},
            "launch_config": ctx.launch_config(), "autotune": tune}
@@ -708,7 +740,8 @@ def main():
     ms_max, ps_all = shard.reduce_measurement(ms, float(ps), dist, "cuda")
     e2e_ms, ps_e2e_all = shard.reduce_measurement(e2e_s * 1e3, float(ps_e2e), dist, "cuda")
 
-    roofline = roofline_of(delta_k, ktimes, ms_k, fused=ctx.launch_config()["grid_step_fused"] > 0)
+    roofline = roofline_of(delta_k, ktimes, ms_k, fused=ctx.launch_config()["grid_step_fused"] > 0,
+                           time_steps=period * args.steps)
 
     line = {
         "metric": METRIC, "value": ps_all / (ms_max * 1e-3), "unit": UNIT,
