@@ -39,7 +39,6 @@ struct Replay {
     float *z[2] = {nullptr, nullptr}, *mu[2] = {nullptr, nullptr};
     uint32_t *id[2] = {nullptr, nullptr}, *pk[2] = {nullptr, nullptr};
     long long *acc[2] = {nullptr, nullptr};
-    uint32_t *stage_l = nullptr;
     unsigned long long *status = nullptr;
     uint32_t *qcnt = nullptr, *fspawn = nullptr;
     DevCounters *cnt = nullptr;
@@ -409,7 +408,7 @@ void free_all(pic_ctx *c)
         r.pk[b] = nullptr;                      // inside r.mu[b]
         release(r.z[b]); release(r.mu[b]); release(r.id[b]); release(r.acc[b]);
     }
-    release(r.stage_l); release(r.status); release(r.qcnt); release(r.fspawn); release(r.cnt); release(r.ctl); release(r.stacks);
+    release(r.status); release(r.qcnt); release(r.fspawn); release(r.cnt); release(r.ctl); release(r.stacks);
     release(r.aent); release(r.aT); release(r.g_ent); release(r.g_T); release(r.gpot);
     release(r.gen_max); release(r.absmax); release(r.qgn); release(r.tot); release(r.parent);
     release(r.gen);
@@ -735,7 +734,7 @@ pic_status pic_init(pic_ctx **out, const pic_params *p, const pic_stack_desc *st
         a.z[b] = c->d_z[b]; a.mu[b] = c->d_mu[b]; a.id[b] = c->d_id[b]; a.pk[b] = c->d_pk[b];
         a.mp_stride = 2;
     }
-    a.stage = c->d_stage;
+    a.stage = reinterpret_cast<float2 *>(c->d_stage);
     a.spawn_bits = c->d_bits;
     a.qrec = c->d_qrec;
     a.n_hist = c->d_nh; a.J_hist = c->d_J; a.cnt = c->d_cnt; a.ctl = c->d_ctl;
@@ -1836,7 +1835,6 @@ pic_status pic_grad(pic_ctx *c, const float *grad_n, const float *grad_J, double
             if (e == cudaSuccess) r.pk[b] = reinterpret_cast<uint32_t *>(r.mu[b]) + 1;
             RALLOC(r.acc[b], c->total_slots);
         }
-        RALLOC(r.stage_l, c->total_slots);
         RALLOC(r.cnt, S); RALLOC(r.ctl, 1); RALLOC(r.stacks, S);
         RALLOC(r.aent, c->n_ent); RALLOC(r.aT, c->n_T);
         RALLOC(r.g_ent, c->n_ent); RALLOC(r.g_T, c->n_T);
@@ -1921,7 +1919,7 @@ pic_status pic_grad(pic_ctx *c, const float *grad_n, const float *grad_J, double
     a.nhw = nullptr; a.bdw = nullptr; a.Jw = nullptr;
     a.tot = r.tot; a.parent = r.parent; a.gen = r.gen; a.gen_max = r.gen_max;
     a.aent = r.aent; a.aT = r.aT; a.g_ent = r.g_ent; a.g_T = r.g_T;
-    a.gn = grad_n ? r.qgn : nullptr; a.gpot = r.gpot; a.stage_l = r.stage_l;
+    a.gn = grad_n ? r.qgn : nullptr; a.gpot = r.gpot;
     a.n_out = n_out; a.ncm = ncm;
 
     // fixed-point scale 2^F: the largest weight maps to at most 2^30 (an

@@ -142,7 +142,7 @@ struct Args {            // everything a kernel needs, passed by value
     uint32_t *id[2];
     uint32_t *pk[2];
     int mp_stride;
-    float4 *stage;
+    float2 *stage;                           // (z, k | layer << 9 | gen << 13) of secondaries without a slot
     unsigned long long *status;      // one look-back word per block
     uint32_t *n_hist;
     // generation labels summed per [stack][n_out][n_cells], at n_off / (2 n_e)
@@ -201,7 +201,6 @@ struct Args {            // everything a kernel needs, passed by value
     double *g_T;                             // gradient, T_thr indexing
     const int32_t *gn;                       // density weights [stack][n_out][2][n_e][ncm]
     const long long *gpot;                   // flux potential [stack][n_out][2][ncm]
-    uint32_t *stage_l;                       // pass 2: start layer of a staged secondary
     int n_out, ncm;                          // moment windows, cells of the widest stack
     double inv_q;                            // 2^-F: reward units to weight units
     // velocity moment [stack][n_out][2][n_cells] at n_off / n_e, units of

@@ -653,25 +653,14 @@ __device__ __forceinline__ void event_item(const Args &a, const DevStack &st, co
                     if (a.flags & PIC_F_STRICT_CAPACITY)
                         atomicCAS(&a.ctl->status, 0u, (unsigned int)PIC_ERR_CAPACITY);
                 } else {
-                    // secondary: same place, spin from P0, isotropic
-                    const uint4 y = philox_rk(make_uint4(key_x, S.ctr_hi, step, SUB_SEC), a);
+                    // secondary: same place; k_place draws its spin and
+                    // direction and flies its half step, a thread per
+                    // secondary (here a few lanes of a warp would do so while
+                    // the others wait)
                     const uint32_t g0 = (pk >> 13) & 0xFFu;
-                    const int sgs = y.x < S.p0[layer] ? 0 : 1;
                     const uint32_t gen = g0 < 255u ? g0 + 1u : 255u;
-                    float zs = z, mus = mu_of(y.y), los = lo, his = hi;
-                    int ls = layer;
-                    TabEnt es = S.ent[(ls * 2 + sgs) * S.n_e + (ks - 1)];
-                    Tally ts{};
-                    flight<DET>(a, S, zs, mus, ls, es, los, his, sgs, ks, half, key_x,
-                                S.ctr_hi, step, SUB_SIF, ts);
-                    // the secondary's boundary events ride in the (not yet
-                    // used) id_hi bits until it is placed
-                    const uint32_t pks = (uint32_t)ks | ((uint32_t)sgs << 8) |
-                                         ((uint32_t)ls << 9) | (gen << 13) |
-                                         (ts.hits << 21) | (ts.trans << 25) |
-                                         (ts.trunc << 29);
-                    a.stage[vpos] = make_float4(zs, mus, __uint_as_float(pks), z);
-                    if (ADJ == 2) a.stage_l[vpos] = (uint32_t)layer;
+                    a.stage[vpos] = make_float2(z, __uint_as_float((uint32_t)ks | ((uint32_t)layer << 9) |
+                                                                   (gen << 13)));
                     atomicOr(&a.spawn_bits[vpos >> 5], 1u << (vpos & 31));
                     atomicAdd(&a.fspawn[f], 1u);
                 }
@@ -1670,56 +1659,6 @@ __device__ __forceinline__ void phase_place(const Args &a)
     const uint32_t *PK = a.pk[cur];
     Tally ty{};
 
-    // Adjoint bookkeeping of a secondary placed at slot d with id `id`, staged
-    // at tile-space position pos (its parent's position).  Pass 1 records the
-    // parent and starts the secondary's own reward with its birth step; pass
-    // 2 flies the secondary's first half step again (the same words) to add
-    // its interface scores weighted by its lineage total, which it still has
-    // to earn and which its parent has now earned.
-    auto place_adj = [&](int s, const DevStack &stg, long long pos, long long d,
-                         unsigned long long id, uint32_t pk, int sg, int k, int c0, int c1,
-                         const float4 &r) {
-        const long long pslot = stg.base + pos - s_tpref[s] * TILE;
-        const uint32_t ppk = PK[2 * pslot], pid_lo = a.id[cur][pslot];
-        const unsigned long long pid = (unsigned long long)pid_lo | ((unsigned long long)(ppk >> 21) << 32);
-        if (id >= (unsigned long long)stg.n_ids || pid >= (unsigned long long)stg.n_ids) {
-            atomicCAS(&a.ctl->status, 0u, (unsigned int)PIC_ERR_STATE);
-            return;
-        }
-        long long rw = flux_w(a, s, tj, sg, c0, c1);
-        if (DEPN) rw += dep_w(a, s, tout, sg, k, c1);
-        if (ADJ == 1) {
-            const unsigned int depth = (unsigned int)a.gen[stg.id_off + pid] + 1u;
-            a.parent[stg.id_off + id] = (unsigned long long)(stg.id_off + pid);
-            a.gen[stg.id_off + id] = (uint8_t)depth;
-            atomicMax(a.gen_max, depth);
-            a.acc[cur][d] = rw;
-        } else {
-            const long long Rc = a.tot[stg.id_off + id];
-            const uint32_t key_x = (uint32_t)(pos - s_tpref[s] * TILE);   // the parent's slot
-            const uint32_t key_y = (uint32_t)(a.stack_base + s) << 16;
-            const uint4 y = philox_rk(make_uint4(key_x, key_y, step, SUB_SEC), a);
-            Stk gs;
-            gs.ent = a.ent + stg.ent_off; gs.T = a.T_thr + stg.T_off;
-            gs.edge = a.stacks[s].edge; gs.p0 = nullptr;
-            gs.n_layers = stg.n_layers; gs.n_cells = stg.n_cells; gs.n_e = a.n_e;
-            gs.ctr_hi = (uint32_t)(a.stack_base + s) << 16; gs.aT = a.aT + stg.T_off;
-            int ls = (int)a.stage_l[pos];
-            TabEnt es = gs.ent[(ls * 2 + sg) * a.n_e + (k - 1)];
-            float los = gs.edge[ls], his = gs.edge[ls + 1];
-            float zs = r.w, mus = mu_of(y.y);
-            Tally tq{};
-            flight<DET, true>(a, gs, zs, mus, ls, es, los, his, sg, k, half, key_x, key_y,
-                              step, SUB_SIF, tq, (double)Rc * a.inv_q, a.g_T + stg.T_off);
-            // the same words give the same flight: anything else means the
-            // replay is not the forward run
-            if (__float_as_uint(zs) != __float_as_uint(r.x))
-                atomicCAS(&a.ctl->status, 0u, (unsigned int)PIC_ERR_STATE);
-            a.acc[cur][d] = Rc - rw;
-            a.acc[cur][pslot] -= Rc;
-        }
-    };
-
     // Place the staged secondaries of stack s in tiles [tl0, tl1) in slot
     // order, the first with rank `prefix` among the stack's secondaries of
     // this step; clears the bitmap words it reads; deposits into the shared
@@ -1731,8 +1670,12 @@ __device__ __forceinline__ void phase_place(const Args &a)
         const unsigned long long nid = a.cnt[s].next_id;
         const int nf = stg.n_cells + 1;
         uint32_t kept = 0;
-        Stk tmp;
-        tmp.n_cells = stg.n_cells;
+        Stk S{};                            // tables read through the caches
+        S.ent = a.ent + stg.ent_off; S.T = a.T_thr + stg.T_off;
+        S.edge = a.stacks[s].edge; S.p0 = a.stacks[s].p0_thr;
+        S.n_layers = stg.n_layers; S.n_cells = stg.n_cells; S.n_e = a.n_e;
+        S.ctr_hi = (uint32_t)(a.stack_base + s) << 16;
+        S.aT = a.aT ? a.aT + stg.T_off : nullptr;
         long long run = prefix;
         // q consecutive bitmap words per thread: PW where the words left fill
         // the block that way, fewer (down to one) near the end of the range,
@@ -1780,25 +1723,66 @@ __device__ __forceinline__ void phase_place(const Args &a)
                 for (int v = tid; v < here; v += TPB) {
                     const long long pos = wb * 32 + (long long)s_list[v];
                     const long long g = run + b0 + v;
-                    const float4 r = a.stage[pos];
-                    const uint32_t pk_staged = __float_as_uint(r.z);
-                    const uint32_t pk = pk_staged & 0x1FFFFFu;
+                    const float2 r = a.stage[pos];
+                    const uint32_t pk_staged = __float_as_uint(r.y);
+                    const int k = (int)(pk_staged & 0xFFu);
                     if (g < room) {
-                        ty.hits += (pk_staged >> 21) & 0xFu;
-                        ty.trans += (pk_staged >> 25) & 0xFu;
-                        ty.trunc += (pk_staged >> 29) & 0x1u;
                         const unsigned long long id = nid + (unsigned long long)g;
                         const long long d = stg.base + nsl + g;
-                        Z[d] = r.x;
+                        const uint32_t key_x = (uint32_t)(pos - s_tpref[s] * TILE);   // the parent's slot
+                        const long long pslot = stg.base + key_x;
+                        // adjoint: the parent's id; pass 2: the secondary's lineage
+                        // total, which it still has to earn and which its parent
+                        // has now earned, weights its interface draws
+                        unsigned long long pid = 0;
+                        bool known = true;
+                        long long Rc = 0;
+                        if (ADJ) {
+                            pid = (unsigned long long)a.id[cur][pslot] |
+                                  ((unsigned long long)(PK[2 * pslot] >> 21) << 32);
+                            known = id < (unsigned long long)stg.n_ids && pid < (unsigned long long)stg.n_ids;
+                            if (!known) atomicCAS(&a.ctl->status, 0u, (unsigned int)PIC_ERR_STATE);
+                            if (ADJ == 2 && known) Rc = a.tot[stg.id_off + id];
+                        }
+                        // spin from P0, isotropic direction, the rest of the step:
+                        // made here, a thread per secondary, instead of by the few
+                        // lanes of an event batch that have one, and once instead
+                        // of twice in pass 2 (gradient of 800 steps of 1e7 carriers
+                        // 551.6 -> 549.7 ms, of 250 steps of 2e5 29.96 -> 29.69)
+                        const uint4 y = philox_rk(make_uint4(key_x, S.ctr_hi, step, SUB_SEC), a);
+                        int layer = (int)((pk_staged >> 9) & 0xFu);
+                        const int sg = y.x < S.p0[layer] ? 0 : 1;
+                        float z = r.x, mu = mu_of(y.y);
+                        TabEnt e = S.ent[(layer * 2 + sg) * S.n_e + (k - 1)];
+                        float lo = S.edge[layer], hi = S.edge[layer + 1];
+                        flight<DET, ADJ == 2>(a, S, z, mu, layer, e, lo, hi, sg, k, half, key_x, S.ctr_hi, step,
+                                              SUB_SIF, ty, ADJ == 2 ? (double)Rc * a.inv_q : 0.0,
+                                              ADJ == 2 ? a.g_T + stg.T_off : nullptr);
+                        const uint32_t pk = (uint32_t)k | ((uint32_t)sg << 8) | ((uint32_t)layer << 9) |
+                                            (pk_staged & (0xFFu << 13));
+                        Z[d] = z;
                         *reinterpret_cast<uint2 *>(MU + 2 * d) =
-                            make_uint2(__float_as_uint(r.y), pk | ((uint32_t)(id >> 32) << 21));
+                            make_uint2(__float_as_uint(mu), pk | ((uint32_t)(id >> 32) << 21));
                         a.id[cur][d] = (uint32_t)id;
                         ++kept;
-                        const int sg = (int)((pk >> 8) & 1u), k = (int)(pk & 0xFFu);
-                        const int c0 = cell_of(a, tmp, r.w), c1 = cell_of(a, tmp, r.x);
-                        if (ADJ) {
-                            place_adj(s, stg, pos, d, id, pk, sg, k, c0, c1, r);
-                        } else {
+                        const int c0 = cell_of(a, S, r.x), c1 = cell_of(a, S, z);
+                        if (ADJ && known) {
+                            // pass 1 records the parent and starts the secondary's
+                            // own reward with its birth step
+                            long long rw = flux_w(a, s, tj, sg, c0, c1);
+                            if (DEPN) rw += dep_w(a, s, tout, sg, k, c1);
+                            if (ADJ == 1) {
+                                const unsigned int depth = (unsigned int)a.gen[stg.id_off + pid] + 1u;
+                                a.parent[stg.id_off + id] = (unsigned long long)(stg.id_off + pid);
+                                a.gen[stg.id_off + id] = (uint8_t)depth;
+                                atomicMax(a.gen_max, depth);
+                                a.acc[cur][d] = rw;
+                            } else {
+                                a.acc[cur][d] = Rc - rw;
+                                a.acc[cur][pslot] -= Rc;
+                            }
+                        }
+                        if (!ADJ) {
                             // a birth, where the parent created it; the
                             // secondary carries its parent's weight
                             atomicAdd(&s_J[sg * nf + c0], 1);
@@ -1813,16 +1797,14 @@ __device__ __forceinline__ void phase_place(const Args &a)
                                 atomicAdd(&s_n[(sg * a.n_e + (k - 1)) * stg.n_cells + c1], 1u);
                                 atomicAdd(&s_gs[c1], (pk >> 13) & 0xFFu);
                                 if (vmom) {
-                                    const int ls = (int)((pk >> 9) & 0xFu);
-                                    const float v = a.ent[stg.ent_off + (ls * 2 + sg) * a.n_e + (k - 1)].v;
                                     add_u64_split(&s_v[sg * stg.n_cells + c1],
-                                                  (unsigned long long)vel_q(__fmul_rn(v, r.y)));
+                                                  (unsigned long long)vel_q(__fmul_rn(e.v, mu)));
                                 }
                             }
                         }
                     } else {
                         ++ty.spawn_drop;
-                        ty.q_drop += pk & 0xFFu;
+                        ty.q_drop += (uint32_t)k;
                     }
                 }
                 cta_sync();
