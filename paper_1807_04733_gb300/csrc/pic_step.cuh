@@ -11,7 +11,8 @@
 //                      boundary in the step; the others are queued
 //   k_event            the general step for the queued carriers; secondaries
 //                      staged at their parents' positions
-//   k_place            slots and ids of the secondaries, in parent slot order
+//   k_place            makes the secondaries: slots and ids in parent slot order,
+//                      spin, direction and the rest of their step
 //   k_inject(half 1)   Source(dt/2), deposited at moment steps
 //   k_compact          every compact_every steps: stable removal of dead slots
 //
