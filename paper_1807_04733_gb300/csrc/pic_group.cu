@@ -29,6 +29,7 @@
 
 #include <algorithm>
 #include <type_traits>
+#include <vector>
 
 #include "pic_step.cuh"
 
@@ -1431,6 +1432,43 @@ cudaError_t group_fits(size_t smem, int threads, bool *ok)
     return e;
 }
 
+// The shapes that k_group may take, the preferred one first; none: the steps are
+// not grouped.  Every one has TPB threads or more: a block decides the group's
+// span at a barrier of its first TPB threads (group_span).
+struct GroupShape {
+    int m, quads, warps, nd, nj;
+    size_t smem;
+};
+
+// densities deposited inside the groups
+bool group_dep(const Args &a) { return a.moment_every < GROUP_DEP_EVERY && !(a.flags & PIC_F_WEIGHTS); }
+
+std::vector<GroupShape> group_shapes(const Args &a, long long slots, int sms, size_t cap)
+{
+    const int me = a.moment_every;
+    const bool dep = group_dep(a);
+    std::vector<GroupShape> r;
+    // Slots per sub-tile: 1024, so that the 2 % of eventful carriers fill most of
+    // a warp (41.5 ms for 50 steps of 4e8 carriers; 52.9 with 512); 512 beside
+    // the density histograms, which leave room for too few warps otherwise
+    // (batched stacks 171 ms for 50 steps against 251); 256 or 512 where larger
+    // ones would leave warps without any.
+    int quads = dep ? 4 : 8;
+    if (slots < (long long)sms * 12 * 1024) quads = 4;
+    if (slots < (long long)sms * 12 * 512) quads = 2;
+    for (int m = slots <= GROUP_LIST_SLOTS ? GROUP_OPEN : GROUP_OPEN_LARGE; m >= 1; --m) {
+        const int nd = dep ? (me - 1 + m) / me : 0;
+        const int nj = dep ? (me + m - 2) / me + 1 : 1;
+        // too few warps beside the histograms: fewer windows
+        const int least = m == 1 || quads == 8 ? TPB / 32 : quads == 4 ? (m > GROUP_OPEN_LARGE ? 14 : TPB / 32) : 12;
+        for (int w = GW_MAX; w >= least; --w) {
+            const GroupSmem o = group_smem(a, dep, quads, w, nd, nj);
+            if (o.total <= cap) r.push_back({m, quads, w, nd, nj, o.total});
+        }
+    }
+    return r;
+}
+
 }  // namespace
 
 static cudaError_t configure_run(const Args &a, GroupCfg *c);
@@ -1444,45 +1482,27 @@ cudaError_t configure_group(const Args &a, long long slots, GroupCfg *gc)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
     const size_t cap = (size_t)optin - 2048;         // less the kernels' static shared memory
-    const int me = a.moment_every;
-    const bool wts = (a.flags & PIC_F_WEIGHTS) != 0;
     // the edges have to do as half-precision numbers
     if (a.dz * (float)a.gbin_max > 32768.f || a.dz < 1.f / 1024.f) return cudaSuccess;
     GroupCfg c;
-    c.dep = me < GROUP_DEP_EVERY && !wts;
-    // Slots per sub-tile: 1024, so that the 2 % of eventful carriers fill most of
-    // a warp (41.5 ms for 50 steps of 4e8 carriers; 52.9 with 512); 512 beside
-    // the density histograms, which leave room for too few warps otherwise
-    // (batched stacks 171 ms for 50 steps against 251); 256 or 512 where larger
-    // ones would leave warps without any.
-    c.quads = c.dep ? 4 : 8;
-    if (slots < (long long)sms * 12 * 1024) c.quads = 4;
-    if (slots < (long long)sms * 12 * 512) c.quads = 2;
-    for (int m = slots <= GROUP_LIST_SLOTS ? GROUP_OPEN : GROUP_OPEN_LARGE; m >= 1 && !c.ok; --m) {
-        const int nd = c.dep ? (me - 1 + m) / me : 0;
-        const int nj = c.dep ? (me + m - 2) / me + 1 : 1;
-        for (int w = GW_MAX; w >= 4; --w) {
-            const GroupSmem o = group_smem(a, c.dep, c.quads, w, nd, nj);
-            if (o.total > cap) continue;
-            // too few warps beside the histograms: fewer windows
-            if (m > 1 && w < (c.quads == 8 ? 6 : c.quads == 4 ? (m > GROUP_OPEN_LARGE ? 14 : 8) : 12)) break;
-            bool ok = false;
-            if (c.dep) {
-                if (c.quads == 8) e = group_fits<true, 8>(o.total, 32 * w, &ok);
-                else if (c.quads == 4) e = group_fits<true, 4>(o.total, 32 * w, &ok);
-                else e = group_fits<true, 2>(o.total, 32 * w, &ok);
-            } else {
-                if (c.quads == 8) e = group_fits<false, 8>(o.total, 32 * w, &ok);
-                else if (c.quads == 4) e = group_fits<false, 4>(o.total, 32 * w, &ok);
-                else e = group_fits<false, 2>(o.total, 32 * w, &ok);
-            }
-            if (e != cudaSuccess) return e;
-            if (!ok) continue;
-            c.m = m; c.nd = nd; c.nj = nj; c.warps = w; c.smem = o.total;
-            c.grid = sms;
-            c.ok = true;
-            break;
+    c.dep = group_dep(a);
+    for (const GroupShape &x : group_shapes(a, slots, sms, cap)) {
+        bool ok = false;
+        if (c.dep) {
+            if (x.quads == 8) e = group_fits<true, 8>(x.smem, 32 * x.warps, &ok);
+            else if (x.quads == 4) e = group_fits<true, 4>(x.smem, 32 * x.warps, &ok);
+            else e = group_fits<true, 2>(x.smem, 32 * x.warps, &ok);
+        } else {
+            if (x.quads == 8) e = group_fits<false, 8>(x.smem, 32 * x.warps, &ok);
+            else if (x.quads == 4) e = group_fits<false, 4>(x.smem, 32 * x.warps, &ok);
+            else e = group_fits<false, 2>(x.smem, 32 * x.warps, &ok);
         }
+        if (e != cudaSuccess) return e;
+        if (!ok) continue;
+        c.m = x.m; c.quads = x.quads; c.warps = x.warps; c.nd = x.nd; c.nj = x.nj; c.smem = x.smem;
+        c.grid = sms;
+        c.ok = true;
+        break;
     }
     if (!c.ok) return cudaSuccess;
     c.smem_tail = (size_t)a.tab_max * sizeof(TabEnt) + (size_t)a.T_max * 4 + 16;
@@ -1572,6 +1592,7 @@ cudaError_t launch_run(const Args &a, const GroupArgs &g, const GroupCfg &c, boo
 cudaError_t launch_group(const Args &a, const GroupArgs &g, const GroupCfg &c, bool det, cudaStream_t s)
 {
     const int nt = 32 * c.warps;
+    if (nt < TPB) return cudaErrorInvalidConfiguration;
 #define PIC_GROUP_LAUNCH(DEP, Q)                                                                   \
     do {                                                                                           \
         if (det) k_group<true, DEP, Q><<<c.grid, nt, c.smem, s>>>(a, g);                           \
@@ -1618,3 +1639,30 @@ cudaError_t launch_mark_base(DevCtl *ctl, cudaStream_t s)
 }
 
 }  // namespace pic
+
+// The shapes of a context of n_stacks stacks with `slots` slots in all and at
+// most `layers` layers and `cells` cells each, from the preferred one: up to
+// `most` of (m, quads, warps) into out; their number.  For checks without a
+// device.
+extern "C" int pic_group_shapes(int n_stacks, int n_e, int layers, int cells, int moment_every, unsigned int flags,
+                                long long slots, int sms, long long smem, int *out, int most)
+{
+    using namespace pic;
+    Args a{};
+    int kb = 0;
+    while ((1 << kb) < n_e + 1) ++kb;
+    a.n_stacks = n_stacks; a.n_e = n_e; a.moment_every = moment_every; a.flags = flags;
+    a.ftab_max = layers * 2 << kb;
+    a.tab_max = layers * 2 * n_e;
+    a.T_max = std::max((layers - 1) * 4 * n_e, 1);
+    a.nbin_max = 2 * n_e * cells;
+    a.gbin_max = cells;
+    a.jbin_max = 2 * (cells + 1);
+    const std::vector<GroupShape> v = group_shapes(a, slots, sms, (size_t)smem);
+    for (int i = 0; i < (int)v.size() && i < most; ++i) {
+        out[3 * i] = v[i].m;
+        out[3 * i + 1] = v[i].quads;
+        out[3 * i + 2] = v[i].warps;
+    }
+    return (int)v.size();
+}

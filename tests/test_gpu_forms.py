@@ -1,0 +1,25 @@
+"""The forms of the step that the context's sizes and tables choose, against
+single steps with a separate event pass (event_pass 1): bit-identical records,
+moments and ledgers (deterministic build)."""
+import numpy as np
+import pytest
+
+from paper_1807_04733_gb300 import pic
+from paper_1807_04733_gb300 import workloads as W
+
+from .test_gpu_group import check, hot, outcome, records
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+DET = W.FLAG_DETERMINISTIC
+
+
+@pytest.mark.parametrize("cells", [260, 315])
+@pytest.mark.parametrize("me", [1, 3])
+def test_large_density_grid(cells, me):
+    """Grids whose density histograms leave room for eight warps (260 cells of
+    60 bins) and for fewer, with the slots of many sub-tiles."""
+    wl = W.bilayer(fe_nm=15, au_nm=cells - 15, n0=300_000, capacity=1_200_000, n_e=60,
+                   n_steps=130, moment_every=me, flags=DET)
+    assert check(wl, [101, 1, 28])[3]["eventful"] > 0
