@@ -739,30 +739,37 @@ __device__ __forceinline__ void agg_sum(unsigned long long *p, uint32_t v)
 // Barrier of the stack's nb blocks (all resident: a cooperative launch) in two
 // halves, between which a block works on what needs no other block: one
 // counter that only grows, `target` the arrivals that end this barrier.  One
-// trip to memory to arrive, then polls; bounded in polls.
+// trip to memory to arrive, then polls; bounded in polls.  The second half is
+// false, for the whole block, where the wait was given up: the lists and counts
+// that it waited for cannot be read.
 __device__ __forceinline__ void stack_arrive(unsigned int *bar)
 {
     cta_sync();
     if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
 }
 
-__device__ __forceinline__ void stack_wait(const Args &a, unsigned int *bar, unsigned int target)
+__device__ __forceinline__ bool stack_wait(const Args &a, unsigned int *bar, unsigned int target)
 {
+    bool given_up = false;
     if (threadIdx.x == 0) {
         unsigned int it = 0, v;
         for (;;) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
             if ((int)(v - target) >= 0) break;
             if (++it > a.spin_limit) {
-                atomicCAS(&a.ctl->status, 0u, (unsigned int)PIC_ERR_TIMEOUT);
+                atomicMax(&a.ctl->status, (unsigned int)PIC_ERR_TIMEOUT);
                 a.ctl->timeout_where = 7u;
+                given_up = true;
                 break;
             }
-            if ((it & 63u) == 0 && *(volatile unsigned int *)&a.ctl->status == (unsigned int)PIC_ERR_TIMEOUT) break;
+            if ((it & 63u) == 0 && timed_out(a)) {
+                given_up = true;
+                break;
+            }
             if (it > 1024) __nanosleep(128);
         }
     }
-    cta_sync();
+    return !cta_sync_or(given_up);
 }
 
 struct TailChild {                   // a secondary before its slot is known
@@ -982,7 +989,7 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
             if (tid < tot0) ch = record(j, u0, tid);
         };
         prepare(0);
-        stack_wait(a, bar, bar_t += (unsigned int)nbk);
+        if (!stack_wait(a, bar, bar_t += (unsigned int)nbk)) return;
         if (tid < GROUP_OPEN) s_tot[tid] = 0u;
         cta_sync();
         for (int i = tid; i < nbk * sp.len; i += TPB) {
@@ -1111,7 +1118,7 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
                 cta_sync();
                 if (tid == 0) g.tsum[(long long)(b0 + ib) * GROUP_OPEN + j] = s_tt[0];
                 stack_arrive(bar);
-                stack_wait(a, bar, bar_t += (unsigned int)nbk);
+                if (!stack_wait(a, bar, bar_t += (unsigned int)nbk)) return;
                 if (tid == 0) s_tt[0] = 0u;
                 cta_sync();
                 for (int b = tid; b < nbk; b += TPB) {
@@ -1212,7 +1219,7 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
             if (j + 1 < sp.len) {
                 if (nsl > n0) stack_arrive(bar); else cta_sync();
                 prepare(j + 1);
-                if (nsl > n0) stack_wait(a, bar, bar_t += (unsigned int)nbk);
+                if (nsl > n0 && !stack_wait(a, bar, bar_t += (unsigned int)nbk)) return;
             }
         }
         // ---- the block's counts
@@ -1383,9 +1390,9 @@ __global__ void __launch_bounds__(32 * GW_MAX, 1) k_run(const Args a, const Grou
     uint32_t s = __ldcg(&a.ctl->step);
     const uint32_t end = s + (uint32_t)n_steps, me = (uint32_t)a.moment_every, ce = (uint32_t)a.compact_every;
     const bool low = threadIdx.x < TPB;
-    auto failed = [&]() -> bool {            // a decision of the whole block
-        return __syncthreads_or(threadIdx.x == 0 && *(volatile unsigned int *)&a.ctl->status != 0u) != 0;
-    };
+    // (decisions of the whole block; a status other than a given-up wait's changes
+    // nothing here, as in single launches)
+    if (__syncthreads_or(threadIdx.x == 0 && timed_out(a))) return;
     while (s < end) {
         uint32_t e = (s / ce + 1) * ce;
         if (e > s + GROUP_MAX) e = s + GROUP_MAX;
@@ -1394,26 +1401,29 @@ __global__ void __launch_bounds__(32 * GW_MAX, 1) k_run(const Args a, const Grou
         while (s < e) {
             const bool no_src = s >= (uint32_t)src_end;
             const Span sp = block_span<DEP>(a, s, (int)(e - s), group_part((int)(e - s), g.m), no_src);
-            if (sp.len == 0) return;         // (never: the step is this launch's own)
+            if (sp.len == 0) return;         // (only after a wait was given up in k_tail's part)
             phase_group<DET, DEP, Q>(a, g, sp);
-            grid_sync(a);
+            if (!grid_sync(a)) return;
             if (low) phase_tail<DET>(a, g, sp, no_src);
-            grid_sync(a);
-            if (failed()) return;
+            if (!grid_sync(a)) return;
             s += (uint32_t)sp.len;
         }
         if (!DEP && e % me == 0) {
             phase_dens(a);
-            if (e < end || e % ce == 0) grid_sync(a);
+            if ((e < end || e % ce == 0) && !grid_sync(a)) return;
         }
         if (e % ce == 0) {
             if (low) phase_compact<0>(a);
-            if (e < end) grid_sync(a);
+            if (e < end && !grid_sync(a)) return;
         }
     }
 }
 
-__global__ void k_mark_base(DevCtl *ctl) { ctl->base = ctl->step; }
+// (after a wait was given up no group of the graph finds its first step)
+__global__ void k_mark_base(DevCtl *ctl)
+{
+    ctl->base = ctl->status == (unsigned int)PIC_ERR_TIMEOUT ? 0x80000000u : ctl->step;
+}
 
 size_t dens_smem(const Args &a)
 {

@@ -551,49 +551,46 @@ __device__ __forceinline__ bool any_source(const Args &a, long long h)
 template <bool DET, bool WSM>
 __global__ void __launch_bounds__(stream_threads<8>(), 2) k_period(const Args a, int n_steps)
 {
-    __shared__ int s_stop;
     const bool low = threadIdx.x < TPB;      // the warps of the 256-thread passes
     for (int i = 0; i < n_steps; ++i) {
-        // stop after a failure (a decision of the whole block)
-        if (threadIdx.x == 0) s_stop = *(volatile unsigned int *)&a.ctl->status != 0u;
-        __syncthreads();
-        if (s_stop) break;
+        // stop after a wait was given up (a decision of the whole block)
+        if (__syncthreads_or(threadIdx.x == 0 && timed_out(a))) return;
         const uint32_t s = __ldcg(a.step_dev);
         const bool dep = ((s + 1) % (uint32_t)a.moment_every) == 0;
         if (any_source(a, 2 * (long long)s)) {
             if (low) phase_inject<0>(a, 0, 0);
-            grid_sync(a);
+            if (!grid_sync(a)) return;
         }
         if (dep) phase_stream<DET, true, false, 8>(a);
         else phase_stream<DET, false, false, 8>(a);
-        grid_sync(a);
+        if (!grid_sync(a)) return;
         if (low) {
             if (dep) phase_event<DET, true>(a);
             else phase_event<DET, false>(a);
         }
-        grid_sync(a);
+        if (!grid_sync(a)) return;
         if (low) {
             if (dep) phase_place<DET, true>(a);
             else phase_place<DET, false>(a);
         }
-        grid_sync(a);
+        if (!grid_sync(a)) return;
         if (any_source(a, 2 * (long long)s + 1)) {
             if (low) phase_inject<0>(a, 1, dep ? 1 : 0);
-            grid_sync(a);
+            if (!grid_sync(a)) return;
         }
         if (dep && a.w[0]) {
             if (low) phase_wdep<WSM>(a, s);
-            grid_sync(a);
+            if (!grid_sync(a)) return;
         }
         if (((s + 1) % (uint32_t)a.compact_every) == 0) {
             if (low) phase_compact<0>(a);
-            grid_sync(a);
+            if (!grid_sync(a)) return;
         }
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             *const_cast<unsigned int *>(a.step_dev) = s + 1u;
             __threadfence();
         }
-        grid_sync(a);
+        if (!grid_sync(a)) return;
     }
 }
 
@@ -668,7 +665,12 @@ cudaError_t launch_inject(const Args &a, const LaunchCfg &c, int half, bool depo
     return cudaGetLastError();
 }
 
-__global__ void k_set_step(DevCtl *ctl, unsigned int step) { ctl->step = ctl->base = step; }
+// (after a wait was given up the step stays where it was: no group's launch
+// finds its first step again)
+__global__ void k_set_step(DevCtl *ctl, unsigned int step)
+{
+    if (ctl->status != (unsigned int)PIC_ERR_TIMEOUT) ctl->step = ctl->base = step;
+}
 
 cudaError_t launch_set_step(DevCtl *ctl, unsigned int step, cudaStream_t s)
 {

@@ -358,6 +358,13 @@ static __device__ long long look_back_warp(const Args &a, unsigned int ep, long 
     return prefix;
 }
 
+// A wait of this context has been given up: it does nothing more until a
+// checkpoint is loaded.
+__device__ __forceinline__ bool timed_out(const Args &a)
+{
+    return *(volatile unsigned int *)&a.ctl->status == (unsigned int)PIC_ERR_TIMEOUT;
+}
+
 // Per-block plan shared by the streaming kernels: tiles of every stack
 // concatenated; this block owns tiles [t0, t1).
 struct Plan {
@@ -2291,9 +2298,13 @@ __global__ void __launch_bounds__(TPB, 4) k_compact(const Args a)
 
 // Grid barrier: every block resident (a cooperative launch).  Sense by
 // generation; the wait is bounded in polls, after which the status says
-// PIC_ERR_TIMEOUT and every later barrier of the launch passes at once.
-__device__ __forceinline__ void grid_sync(const Args &a)
+// PIC_ERR_TIMEOUT.  False, for the whole block: the wait was given up (here or by
+// another block), what the barrier was to order cannot be read, and the block
+// has to leave the launch.  Any other status, such as a full buffer's, changes
+// nothing: the passes go on as single launches do.
+__device__ __forceinline__ bool grid_sync(const Args &a)
 {
+    int given_up = 0;
     __syncthreads();
     if (threadIdx.x == 0) {
         volatile unsigned int *gen = &a.ctl->bar_gen;
@@ -2306,10 +2317,14 @@ __device__ __forceinline__ void grid_sync(const Args &a)
         } else {
             unsigned int it = 0;
             while (*gen == g) {
-                if (*(volatile unsigned int *)&a.ctl->status != 0u) break;
+                if (timed_out(a)) {
+                    given_up = 1;
+                    break;
+                }
                 if (++it > a.spin_limit) {
-                    atomicCAS(&a.ctl->status, 0u, (unsigned int)PIC_ERR_TIMEOUT);
+                    atomicMax(&a.ctl->status, (unsigned int)PIC_ERR_TIMEOUT);
                     a.ctl->timeout_where = 5u;
+                    given_up = 1;
                     break;
                 }
                 if (it > 64) __nanosleep(256);
@@ -2317,7 +2332,7 @@ __device__ __forceinline__ void grid_sync(const Args &a)
         }
         __threadfence();
     }
-    __syncthreads();
+    return __syncthreads_or(given_up) == 0;
 }
 
 // ---------------------------------------------------------------------------
