@@ -1084,6 +1084,9 @@ cudaError_t enqueue_range(pic_ctx *c, const Args &a0, int s, int e, const unsign
     Args a = a0;
     a.step_dev = &c->d_ctl->step;
     a.bump_step = 0;
+    a.due = 1;
+    a.due_step = (uint32_t)e;
+    a.due_base = base;
     GroupArgs g = c->ga;
     g.base = base;
     g.end = e;

@@ -1375,7 +1375,7 @@ __device__ __forceinline__ void phase_dens(const Args &a)
 
 __global__ void __launch_bounds__(DENS_T) k_dens(const Args a)
 {
-    phase_dens(a);
+    if (range_done(a)) phase_dens(a);
 }
 
 // ---------------------------------------------------------------------------

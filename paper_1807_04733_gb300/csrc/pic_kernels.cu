@@ -245,7 +245,7 @@ __device__ __forceinline__ void phase_wdep(const Args &a, uint32_t step)
 template <bool SM>
 __global__ void __launch_bounds__(TPB) k_wdep(const Args a)
 {
-    phase_wdep<SM>(a, a.step_dev ? __ldcg(a.step_dev) - 1u : a.step);
+    if (range_done(a)) phase_wdep<SM>(a, a.step_dev ? __ldcg(a.step_dev) - 1u : a.step);
 }
 
 // What a reading call takes to the host: a stack's counters and the device

@@ -365,6 +365,14 @@ __device__ __forceinline__ bool timed_out(const Args &a)
     return *(volatile unsigned int *)&a.ctl->status == (unsigned int)PIC_ERR_TIMEOUT;
 }
 
+// Whether the grouped steps before this launch have come to the end of their
+// range (they have not after a given-up wait: the window and the state that the
+// launch is for are not there).  Uniform over the grid.
+__device__ __forceinline__ bool range_done(const Args &a)
+{
+    return !a.due || __ldcg(&a.ctl->step) == (a.due_base ? __ldcg(a.due_base) : 0u) + a.due_step;
+}
+
 // Per-block plan shared by the streaming kernels: tiles of every stack
 // concatenated; this block owns tiles [t0, t1).
 struct Plan {
@@ -2293,7 +2301,7 @@ __device__ __forceinline__ void phase_compact(const Args &a)
 template <int ADJ = 0>
 __global__ void __launch_bounds__(TPB, 4) k_compact(const Args a)
 {
-    phase_compact<ADJ>(a);
+    if (range_done(a)) phase_compact<ADJ>(a);
 }
 
 // Grid barrier: every block resident (a cooperative launch).  Sense by

@@ -63,3 +63,18 @@ def test_steps_go_on_after_an_overflow(me, graph):
         assert x[0] == 3 and x[1]["spawn_dropped"] > 0
     a.close()
     b.close()
+
+
+def test_windows_after_an_overflow_inside_one():
+    """Windows of 50 steps that calls of different lengths end, a whole group's
+    launch and a short one's, after an overflow within the first window."""
+    wl = overflowing(50, ce=40)
+    a, b = begin(wl), begin(wl, event_pass=1)
+    for n in (45, 5, 47, 3, 100, 50):
+        a.step(n)
+        b.step(n)
+    same(moments(a, wl), moments(b, wl))
+    for s in range(2):
+        assert torch.equal(a.gen_moments(s), b.gen_moments(s))
+    a.close()
+    b.close()
