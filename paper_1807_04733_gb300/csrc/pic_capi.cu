@@ -439,6 +439,18 @@ cudaError_t timed(pic_ctx *c, int kind, F fn)
     return e;
 }
 
+// The grouped steps' counts as before a first step: no launch is in flight.
+cudaError_t reset_groups(pic_ctx *c)
+{
+    if (!c->gc.ok) return cudaSuccess;
+    cudaError_t e = cudaMemsetAsync(c->d_gabs, 0, sizeof(uint32_t) * (size_t)c->n_stacks * GROUP_MAX, c->stream);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(c->d_gbar, 0, sizeof(unsigned int) * 32 * (size_t)c->n_stacks, c->stream);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(c->d_gcnt, 0, sizeof(uint16_t) * (size_t)GROUP_OPEN * (size_t)c->ga.cnt_n, c->stream);
+    return e;
+}
+
 // First step after which no stack's source creates a carrier.
 int source_end(const pic_ctx *c)
 {
@@ -874,8 +886,7 @@ pic_status pic_init(pic_ctx **out, const pic_params *p, const pic_stack_desc *st
     DevCtl ctl{};
     ctl.epoch = 1u;
     if (c->gc.ok) {
-        e = cudaMemsetAsync(c->d_gabs, 0, sizeof(uint32_t) * (size_t)n_stacks * GROUP_MAX, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->d_gbar, 0, sizeof(unsigned int) * 32 * (size_t)n_stacks, st);
+        e = reset_groups(c);
         if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_gblk, blk.data(), sizeof(int4) * blk.size(), cudaMemcpyHostToDevice, st);
     }
     std::vector<DevCounters> cnt(n_stacks);
@@ -1523,6 +1534,7 @@ pic_status pic_load(pic_ctx *c, const void *buf, size_t bytes)
     if (e == cudaSuccess)
         e = cudaMemsetAsync(c->d_status, 0, sizeof(unsigned long long) * c->n_words, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_fspawn, 0, sizeof(uint32_t) * c->n_status, c->stream);
+    if (e == cudaSuccess) e = reset_groups(c);    // (a launch that gave up a wait leaves them as they were)
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "pic_load copy");
     c->step = hd.step;

@@ -78,3 +78,24 @@ def test_windows_after_an_overflow_inside_one():
         assert torch.equal(a.gen_moments(s), b.gen_moments(s))
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("graph", [0, 1, 2])
+def test_checkpoint_loaded_after_a_failure(graph):
+    """The context steps on from the checkpoint as a fresh one does."""
+    wl = overflowing(5)
+    a = pic.Context(wl, use_graph=graph)
+    a.step(30)
+    blob = a.save()
+    a.set_records(records(wl, 9_001), 9_001)
+    a.step(70)
+    assert moments(a, wl)[0] == 3
+    a.load(blob)
+    b = pic.Context(wl, use_graph=graph)
+    b.load(blob)
+    for n in (20, 70):
+        a.step(n)
+        b.step(n)
+        same(moments(a, wl), moments(b, wl))
+    a.close()
+    b.close()
