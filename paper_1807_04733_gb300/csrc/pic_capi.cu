@@ -1529,6 +1529,10 @@ pic_status pic_load(pic_ctx *c, const void *buf, size_t bytes)
         if (e == cudaSuccess && x.second) e = cudaMemcpyAsync(x.first, o, x.second, cudaMemcpyHostToDevice, c->stream);
         o += x.second;
     }
+    // no fluxes in the windows that the loaded run has not reached
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_J, 0, 4 * (size_t)std::max<int64_t>(c->J_total, 1), c->stream);
+    if (e == cudaSuccess && wts)
+        e = cudaMemsetAsync(c->d_Jw, 0, 8 * (size_t)std::max<int64_t>(c->J_total, 1), c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_cnt, cnt.data(), sizeof(DevCounters) * S, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_ctl, &ctl, sizeof(DevCtl), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess)
