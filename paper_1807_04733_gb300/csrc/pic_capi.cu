@@ -103,6 +103,7 @@ struct pic_ctx {
     // memory takes a third of a millisecond to allocate), else mapped memory
     HostRead h_own{};
     HostRead *h_read = nullptr, *h_read_dev = nullptr;
+    int device = -1;                 // the device of the context's memory
     Args args{};
     LaunchCfg lc{};
     int step = 0;
@@ -484,32 +485,39 @@ pic_status device_status(pic_ctx *c)
     return status_result(c, h.status);
 }
 
-bool on_device(const void *p)
+// Whether a kernel of the context may store words at p: memory of the context's
+// own device, which another device's (peer access may be off), managed and host
+// memory are not, and a word's alignment.
+bool kernel_stores(int type, int device, int ctx_device, uintptr_t p)
+{
+    return type == (int)cudaMemoryTypeDevice && device == ctx_device && p % 4 == 0;
+}
+
+bool kernel_stores(const pic_ctx *c, const void *p)
 {
     cudaPointerAttributes at{};
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return at.type == cudaMemoryTypeDevice;
+    return kernel_stores((int)at.type, at.device, c->device, reinterpret_cast<uintptr_t>(p));
 }
 
-// Ends a reading call: copies n_words and j_words words (destinations in host or
-// device memory; null: none), brings the stack's counters and the device status
-// to the host and waits.  What stays on the device goes with the counters in
-// one launch; they come by mapped host memory, where a copy of each from
-// pageable memory took most of a small call's time.
-pic_status read_out(pic_ctx *c, int stack, const uint32_t *n_src, void *n_dst, size_t n_words,
-                    const uint32_t *j_src, void *j_dst, size_t j_words, DevCounters *hc, const char *where)
+// Ends a reading call: copies n_words and j_words words (null: none), brings the
+// stack's counters and the device status to the host and waits.  The buffers
+// may be any memory that a copy of `kind` takes.  What stays on the context's
+// device goes with the counters in one launch; they come by mapped host memory,
+// where a copy of each from pageable memory took most of a small call's time.
+pic_status read_out(pic_ctx *c, int stack, const uint32_t *n_src, void *n_dst, size_t n_words, const uint32_t *j_src,
+                    void *j_dst, size_t j_words, cudaMemcpyKind kind, DevCounters *hc, const char *where)
 {
     cudaError_t e = cudaSuccess;
     // (a copy engine is as good for large ones)
     const size_t most = 1u << 20;
-    const bool nk = n_dst && n_words && n_words <= most && on_device(n_dst);
-    const bool jk = j_dst && j_words && j_words <= most && on_device(j_dst);
-    if (n_dst && n_words && !nk) e = cudaMemcpyAsync(n_dst, n_src, 4 * n_words, cudaMemcpyDefault, c->stream);
-    if (e == cudaSuccess && j_dst && j_words && !jk)
-        e = cudaMemcpyAsync(j_dst, j_src, 4 * j_words, cudaMemcpyDefault, c->stream);
+    const bool nk = n_dst && n_words && n_words <= most && kernel_stores(c, n_dst);
+    const bool jk = j_dst && j_words && j_words <= most && kernel_stores(c, j_dst);
+    if (n_dst && n_words && !nk) e = cudaMemcpyAsync(n_dst, n_src, 4 * n_words, kind, c->stream);
+    if (e == cudaSuccess && j_dst && j_words && !jk) e = cudaMemcpyAsync(j_dst, j_src, 4 * j_words, kind, c->stream);
     if (e == cudaSuccess)
         e = launch_read(c->d_cnt + stack, c->d_ctl, c->h_read_dev, n_src, static_cast<uint32_t *>(n_dst),
                         nk ? (long long)n_words : 0, j_src, static_cast<uint32_t *>(j_dst),
@@ -719,9 +727,9 @@ pic_status pic_init(pic_ctx **out, const pic_params *p, const pic_stack_desc *st
     ALLOC(c->d_hnow, (size_t)n_stacks * 2 * (c->ncm + 1));
     ALLOC(c->d_cnt, n_stacks);
     ALLOC(c->d_ctl, 1);
-    int dev_id = 0, pageable = 0;
-    if (e == cudaSuccess) e = cudaGetDevice(&dev_id);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, dev_id);
+    int pageable = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&c->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, c->device);
     if (e == cudaSuccess && pageable) {
         c->h_read = c->h_read_dev = &c->h_own;
     } else {
@@ -1568,7 +1576,7 @@ pic_status pic_moments(pic_ctx *c, int stack, uint32_t *n_dev, int32_t *J_dev, p
     const size_t nj = (size_t)h.n_out * 2 * (h.n_cells + 1);
     DevCounters hc{};
     const pic_status st = read_out(c, stack, c->d_nh + d.n_off, n_dev, nn, reinterpret_cast<const uint32_t *>(c->d_J + d.J_off),
-                                   J_dev, nj, &hc, "pic_moments copy");
+                                   J_dev, nj, cudaMemcpyDeviceToDevice, &hc, "pic_moments copy");
     if (led) {
         static_assert(sizeof(pic_ledger) == sizeof(unsigned long long) * LEDGER_N, "ledger layout");
         std::memcpy(led, hc.led, sizeof(pic_ledger));
@@ -1591,7 +1599,7 @@ pic_status pic_moment_window(pic_ctx *c, int stack, int window, uint32_t *n_out,
     DevCounters hc{};
     const pic_status st = read_out(c, stack, c->d_nh + d.n_off + (size_t)window * nn, n_out, nn,
                                    reinterpret_cast<const uint32_t *>(c->d_J + d.J_off + (size_t)window * nj), J_out, nj,
-                                   &hc, "pic_moment_window copy");
+                                   cudaMemcpyDefault, &hc, "pic_moment_window copy");
     if (led) std::memcpy(led, hc.led, sizeof(pic_ledger));
     return st;
 }
@@ -2258,6 +2266,12 @@ pic_status pic_autotune(pic_ctx *c, int trial_steps, pic_tune_entry *entries, in
         for (int i = 0; i < (int)res.size() && i < max_entries; ++i) entries[i] = res[i];
     if (n_entries) *n_entries = (int)res.size();
     return PIC_OK;
+}
+
+// kernel_stores of a pointer's attributes, for checks without a device
+int pic_kernel_stores(int type, int device, int ctx_device, uint64_t p)
+{
+    return kernel_stores(type, device, ctx_device, (uintptr_t)p) ? 1 : 0;
 }
 
 pic_status pic_profile(pic_ctx *c, int enable)
