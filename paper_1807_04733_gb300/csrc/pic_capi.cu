@@ -1135,6 +1135,17 @@ cudaError_t enqueue_range(pic_ctx *c, const Args &a0, int s, int e, const unsign
     return r;
 }
 
+// Whether the caller is capturing the context's stream.
+bool capturing(const pic_ctx *c)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st == cudaStreamCaptureStatusActive;
+}
+
 // Whether single launches give way to the persistent form: few carriers, where
 // the gaps between the launches of a group count (a run of 500 steps from 1e5
 // carriers 9.1 -> 8.4 ms, one of 600 steps from 1.2e6 carriers 28.8 -> 28.4;
@@ -1249,6 +1260,10 @@ pic_status pic_step(pic_ctx *c, int n_steps)
         const long long l = (long long)me / gcd_int(me, ce) * ce;
         c->period = l <= 100000 ? (int)l : -1;      // -1: no graphs for this context
     }
+    // Launches that a caller captures name their steps themselves: they are these
+    // steps at every replay, and the device step is no longer known here.
+    const bool cap = grouped(c) && capturing(c);
+    if (cap && !graphs) c->dev_step_valid = false;
     int left = n_steps;
     while (left > 0) {
         const int s = c->step;
@@ -1348,6 +1363,7 @@ pic_status pic_step(pic_ctx *c, int n_steps)
         c->step = s + 1;
         --left;
     }
+    if (cap && !graphs) c->dev_step_valid = false;
     return PIC_OK;
 }
 
