@@ -281,6 +281,8 @@ struct LaunchCfg {
     int grid_slow, grid_slow_dep;          // k_event
     int grid_place, grid_place_dep;        // k_place
     int grid_compact, grid_inject;
+    int grid_wdep;                         // weighted densities, and their shared memory
+    size_t smem_wdep;                      //   (0: added in global memory)
     int ring_fast, ring_fast_dep;
     size_t smem_fast, smem_fast_dep, smem_slow, smem_slow_dep, smem_place, smem_place_dep;
     // the fused streaming pass (plain steps of a single stack; grid 0: not used)

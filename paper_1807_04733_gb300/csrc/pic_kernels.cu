@@ -298,20 +298,8 @@ cudaError_t launch_state_hist_w(const Args &a, int s0, int s1, int mode, int win
 
 cudaError_t launch_wdep(const Args &a, const LaunchCfg &c, cudaStream_t st)
 {
-    // privatised in shared memory when the widest stack's histogram fits
-    const size_t sm = (size_t)a.nbin_max * sizeof(unsigned long long);
-    int dev = 0, optin = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e != cudaSuccess) return e;
-    const size_t static_sm = (size_t)(2 * PIC_MAX_STACKS + 1) * 8;
-    if (sm + static_sm <= (size_t)optin) {
-        e = cudaFuncSetAttribute(k_wdep<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        k_wdep<true><<<c.grid_compact, TPB, sm, st>>>(a);
-    } else {
-        k_wdep<false><<<c.grid_compact, TPB, 0, st>>>(a);
-    }
+    if (c.smem_wdep) k_wdep<true><<<c.grid_wdep, TPB, c.smem_wdep, st>>>(a);
+    else k_wdep<false><<<c.grid_wdep, TPB, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -444,6 +432,21 @@ cudaError_t configure(const Args &a, int blocks_per_sm, int ring_req, int hist_m
         return e;
     cfg->grid_compact = sms * (oc > 0 ? oc : 1);
     cfg->grid_inject = sms * 4;
+    // The weighted densities: the blocks that are resident beside their
+    // histograms.  (3 per SM for 115 cells of 30 bins: 26 us for 4e6 slots, 204
+    // for 4e7; with the compaction's grid, 4 per SM, 34 and 296.)
+    cfg->grid_wdep = 0;
+    cfg->smem_wdep = 0;
+    if (a.w[0]) {
+        int ow = 0;
+        cfg->smem_wdep = (size_t)a.nbin_max * sizeof(unsigned long long);
+        if ((e = occupancy(k_wdep<true>, cfg->smem_wdep, &ow)) != cudaSuccess) return e;
+        if (ow < 1) {
+            cfg->smem_wdep = 0;
+            if ((e = occupancy(k_wdep<false>, 0, &ow)) != cudaSuccess) return e;
+        }
+        cfg->grid_wdep = sms * std::max(ow, 1);
+    }
     return cudaSuccess;
 }
 
