@@ -878,6 +878,7 @@ pic_status pic_init(pic_ctx **out, const pic_params *p, const pic_stack_desc *st
         g.sub = 128 * c->gc.quads;
         g.nd = c->gc.nd;
         g.nj = c->gc.nj;
+        g.tail_sums = c->gc.tail_sums ? 1 : 0;
         g.m = c->gc.m;
         c->ga_run = g;
         c->ga_run.blk = c->d_gblk + gt;

@@ -785,7 +785,24 @@ struct TailStack {                   // what a tail block keeps of its stack
     float *Z, *MU;
     uint32_t *ID, *W;
     bool vmom;
+    // births minus removals, generation and velocity sums of the group's windows
+    // (from tj0) in shared memory; null: added in memory
+    int tj0;
+    int32_t *J;
+    uint32_t *G;
+    unsigned long long *V;
 };
+
+// Their shared memory.  In memory the sums fall on a few lines (115 cells: 7 lines
+// of generation sums and 8 of births), whose additions one after another were
+// most of what many new carriers cost: k_tail's part of 20 steps of 2e7 carriers
+// that start at 1.5 eV, 1.7e7 secondaries, took 9.0 ms with densities every step
+// (single steps' event and placement passes 5.1) and 4.5 ms without, now 1.9 and 1.4.
+__host__ __device__ inline size_t tail_sums(const Args &a, int nd, int nj)
+{
+    const bool vmom = nd > 0 && (a.flags & PIC_F_VELOCITY_MOMENTS);
+    return (size_t)nj * a.jbin_max * 4 + (size_t)nd * a.gbin_max * (vmom ? 20 : 4) + 8;
+}
 
 // the density, generation and velocity sums of one carrier at the end of window t
 __device__ __forceinline__ void tail_deposit(const Args &a, const TailStack &x, int t, int sg, int k,
@@ -793,19 +810,26 @@ __device__ __forceinline__ void tail_deposit(const Args &a, const TailStack &x, 
 {
     const int c = cell_at(z, a.inv_dz, x.nc);
     agg_add(&a.n_hist[x.st->n_off + ((long long)t * 2 + sg) * x.ne * x.nc + (long long)(k - 1) * x.nc + c], 1);
-    agg_sum(&a.g_hist[x.st->n_off / (2 * x.ne) + (long long)t * x.nc + c], gen);
-    if (x.vmom)
+    if (x.G) atomicAdd(&x.G[(t - x.tj0) * x.nc + c], gen);
+    else agg_sum(&a.g_hist[x.st->n_off / (2 * x.ne) + (long long)t * x.nc + c], gen);
+    if (x.vmom && x.V)
+        add_u64_split(&x.V[((t - x.tj0) * 2 + sg) * x.nc + c], (unsigned long long)vel_q(w));
+    else if (x.vmom)
         atomicAdd(reinterpret_cast<unsigned long long *>(a.v_hist) + x.st->n_off / x.ne +
                       ((long long)t * 2 + sg) * x.nc + c,
                   (unsigned long long)vel_q(w));
 }
 
-// a birth in window t, with its weight
-__device__ __forceinline__ void tail_birth(const Args &a, const TailStack &x, int t, int sg, float z, uint32_t w)
+// a birth (+1) or removal (-1) in window t, with its weight
+__device__ __forceinline__ void tail_change(const Args &a, const TailStack &x, int t, int sg, float z, int by, uint32_t w)
 {
-    const long long i = x.st->J_off + ((long long)t * 2 + sg) * x.nf + cell_at(z, a.inv_dz, x.nc);
-    agg_add(reinterpret_cast<uint32_t *>(&a.bd_hist[i]), 1);
-    if (a.w[0]) atomicAdd(reinterpret_cast<unsigned long long *>(a.bdw) + i, (unsigned long long)w);
+    const int c = cell_at(z, a.inv_dz, x.nc);
+    const long long i = x.st->J_off + ((long long)t * 2 + sg) * x.nf + c;
+    if (x.J) atomicAdd(&x.J[((t - x.tj0) * 2 + sg) * x.nf + c], by);
+    else agg_add(reinterpret_cast<uint32_t *>(&a.bd_hist[i]), by);
+    if (a.w[0])
+        atomicAdd(reinterpret_cast<unsigned long long *>(a.bdw) + i,
+                  by > 0 ? (unsigned long long)w : 0ull - (unsigned long long)w);
 }
 
 // Source(dt/2): the carrier with id `id` in slot `slot`
@@ -853,7 +877,7 @@ __device__ __forceinline__ void tail_source(const Args &a, const TailStack &x, u
         x.W[slot] = wq;
         wsum += wq;
     }
-    tail_birth(a, x, t, (int)sg, z, wq);
+    tail_change(a, x, t, (int)sg, z, 1, wq);
     if (deposit) {
         const float v = x.vmom ? a.ent[st.ent_off + (layer * 2 + sg) * x.ne + (k - 1)].v : 0.f;
         tail_deposit(a, x, t, (int)sg, (int)k, 1u, z, __fmul_rn(v, mu));
@@ -901,6 +925,19 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
         x.ID = a.id[cur] + st.base;
         x.W = a.w[0] ? a.w[cur] + st.base : nullptr;
         x.vmom = (a.flags & PIC_F_VELOCITY_MOMENTS) != 0;
+        x.tj0 = (int)(sp.s0 / me);
+        x.J = nullptr; x.G = nullptr; x.V = nullptr;
+        // (32 bits hold the generation sums of 2^24 carriers)
+        const bool sums = g.tail_sums && st.cap / nbk < (1 << 24);
+        const int nv = sums && x.vmom && g.nd > 0 ? g.nd * 2 * x.nc : 0, nj = sums ? g.nj * 2 * x.nf : 0,
+                  ng = sums ? g.nd * x.nc : 0;
+        if (sums) {
+            x.V = reinterpret_cast<unsigned long long *>((reinterpret_cast<uintptr_t>(s_T + a.T_max) + 7) & ~uintptr_t(7));
+            x.J = reinterpret_cast<int32_t *>(x.V + nv);
+            x.G = reinterpret_cast<uint32_t *>(x.J + nj);
+            for (int i = tid; i < nv; i += TPB) x.V[i] = 0ull;
+            for (int i = tid; i < nj + ng; i += TPB) x.J[i] = 0;
+        }
         const float half = a.half_dt;
         const bool dep_in = g.nd > 0;            // densities deposited inside the group
         const long long U = (n0 + g.sub - 1) / g.sub;      // sub-tiles of the group's start
@@ -1086,11 +1123,7 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
                         }
                         if (dead) {
                             pk = (pk & ~0x1FFFu) | ((uint32_t)sg << 8) | ((uint32_t)layer << 9);
-                            const long long i = st.J_off + ((long long)t * 2 + sg) * x.nf + cell_at(z, a.inv_dz, x.nc);
-                            agg_add(reinterpret_cast<uint32_t *>(&a.bd_hist[i]), -1);
-                            if (a.w[0])
-                                atomicAdd(reinterpret_cast<unsigned long long *>(a.bdw) + i,
-                                          0ull - (unsigned long long)x.W[slot]);
+                            tail_change(a, x, t, sg, z, -1, a.w[0] ? x.W[slot] : 0u);
                             atomicAdd(&g.abs[s * GROUP_MAX + j], 1u);
                         } else {
                             flight<DET>(a, S, z, mu, layer, e, lo, hi, sg, k, half, (uint32_t)slot, x.ctr_hi,
@@ -1166,7 +1199,7 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
                     wp = __ldcg(&x.W[c.pslot]);
                     x.W[d] = wp;
                 }
-                tail_birth(a, x, t, sg, c.zb, wp);
+                tail_change(a, x, t, sg, c.zb, 1, wp);
                 if (dep) tail_deposit(a, x, t, sg, ks, (c.pk >> 13) & 0xFFu, c.z, __fmul_rn(c.v, c.mu));
             };
             if (s_tot[j] > 0) {
@@ -1222,7 +1255,20 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
                 if (nsl > n0 && !stack_wait(a, bar, bar_t += (unsigned int)nbk)) return;
             }
         }
-        // ---- the block's counts
+        // ---- the block's sums and counts
+        if (sums) {
+            cta_sync();
+            int32_t *gJ = a.bd_hist + st.J_off + (long long)x.tj0 * 2 * x.nf;
+            unsigned long long *gG = a.g_hist + st.n_off / (2 * x.ne) + (long long)x.tj0 * x.nc;
+            unsigned long long *gV = reinterpret_cast<unsigned long long *>(a.v_hist) + st.n_off / x.ne +
+                                     (long long)x.tj0 * 2 * x.nc;
+            for (int i = tid; i < nj; i += TPB)
+                if (x.J[i]) atomicAdd(&gJ[i], x.J[i]);
+            for (int i = tid; i < ng; i += TPB)
+                if (x.G[i]) atomicAdd(&gG[i], (unsigned long long)x.G[i]);
+            for (int i = tid; i < nv; i += TPB)
+                if (x.V[i]) atomicAdd(&gV[i], x.V[i]);
+        }
         const uint32_t vals[10] = {ty.absorbed, ty.bath, ty.hits, ty.trans, ty.trunc, ty.spawn_drop,
                                    ty.q_drop, ty.changed, kept_here, (uint32_t)n_event};
         const unsigned long long v = block_sums<10>(vals, s_r8);
@@ -1516,6 +1562,9 @@ cudaError_t configure_group(const Args &a, long long slots, GroupCfg *gc)
     }
     if (!c.ok) return cudaSuccess;
     c.smem_tail = (size_t)a.tab_max * sizeof(TabEnt) + (size_t)a.T_max * 4 + 16;
+    // (two blocks per SM keep theirs beside the tables)
+    c.tail_sums = tail_sums(a, c.nd, c.nj) <= 48 * 1024;
+    if (c.tail_sums) c.smem_tail += tail_sums(a, c.nd, c.nj);
     int o1 = 0, o2 = 0;
     e = occupancy(k_tail<false>, c.smem_tail, &o1);
     if (e == cudaSuccess) e = occupancy(k_tail<true>, c.smem_tail, &o2);

@@ -248,6 +248,7 @@ struct GroupArgs {
     const int4 *blk;             // per tail block: stack, index in it, the stack's blocks, the first
     int sub;                     // slots per sub-tile
     int nd, nj;                  // density and removal windows held in shared memory
+    int tail_sums;               // k_tail holds its sums over cells in shared memory
 };
 
 // Steps of the next group of a range of n: equal parts of at most m.
@@ -262,6 +263,7 @@ inline int group_part(int n, int m)
 
 struct GroupCfg {
     bool ok = false, dep = false;    // dep: densities deposited inside the group
+    bool tail_sums = false;
     int m = 0, quads = 0, warps = 0, nd = 0, nj = 0;
     int grid = 0, grid_tail = 0, grid_dens = 0;
     size_t smem = 0, smem_tail = 0, smem_dens = 0;
