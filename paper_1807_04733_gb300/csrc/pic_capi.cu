@@ -1106,7 +1106,7 @@ cudaError_t enqueue_range(pic_ctx *c, const Args &a0, int s, int e, const unsign
     a.bump_step = 0;
     a.due = 1;
     a.due_step = (uint32_t)e;
-    a.due_base = base;
+    a.due_period = base ? (uint32_t)c->period : 0u;
     GroupArgs g = c->ga;
     g.base = base;
     g.end = e;

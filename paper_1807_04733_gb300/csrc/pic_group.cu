@@ -1345,6 +1345,7 @@ __device__ __forceinline__ void phase_dens(const Args &a)
     long long *s_nsl = s_tpref + a.n_stacks + 1;
     const int tid = threadIdx.x, ne = a.n_e;
     const int cur = (int)__ldcg(&a.ctl->cur);
+    const RangeEnd end(a);
     const int t = (int)(__ldcg(&a.ctl->step) / (uint32_t)a.moment_every) - 1;
     for (int s = tid; s < a.n_stacks; s += NT) s_nsl[s] = (long long)a.cnt[s].n_slots;
     __syncthreads();
@@ -1359,7 +1360,7 @@ __device__ __forceinline__ void phase_dens(const Args &a)
     __syncthreads();
     const long long T = s_tpref[a.n_stacks];
     const long long t0 = chunk_lo(T, blockIdx.x, gridDim.x), t1 = chunk_lo(T, blockIdx.x + 1, gridDim.x);
-    if (t0 >= t1) return;
+    if (t0 >= t1 || !end.reached(a)) return;
     const int s_first = stack_of(s_tpref, a.n_stacks, t0), s_last = stack_of(s_tpref, a.n_stacks, t1 - 1);
     for (int s = s_first; s <= s_last; ++s) {
         const long long ta = t0 > s_tpref[s] ? t0 : s_tpref[s];
@@ -1421,7 +1422,7 @@ __device__ __forceinline__ void phase_dens(const Args &a)
 
 __global__ void __launch_bounds__(DENS_T) k_dens(const Args a)
 {
-    if (range_done(a)) phase_dens(a);
+    phase_dens(a);
 }
 
 // ---------------------------------------------------------------------------

@@ -167,10 +167,10 @@ struct Args {            // everything a kernel needs, passed by value
     const unsigned int *step_dev;            // graph replay: the step is read here
     int bump_step;                           // this kernel's last block advances *step_dev
     // what is due at the end of a range of grouped steps runs only if the device
-    // step is due_step from *due_base (null: from 0); due 0: whatever it is
+    // step is due_step, in graphs (due_period > 0) whole periods after it; due 0:
+    // whatever it is
     int due;
-    uint32_t due_step;
-    const unsigned int *due_base;
+    uint32_t due_step, due_period;
     int tab_max, T_max, nbin_max, jbin_max;  // shared-memory sizing
     int ftab_max;                            // entries of the padded fast table
     int gbin_max;                            // cells of the widest stack (generation sums)

@@ -189,8 +189,10 @@ __device__ __forceinline__ void phase_wdep(const Args &a, uint32_t step)
     const int cur = (int)*(volatile unsigned int *)&a.ctl->cur;
     const int tid = threadIdx.x;
     const int tout = (int)((step + 1) / (uint32_t)a.moment_every) - 1;
+    const RangeEnd end(a);
     Plan p;
     make_plan(a, s_tpref, s_nsl, p);
+    if (!end.reached(a)) return;
     const uint2 *MP = reinterpret_cast<const uint2 *>(a.mu[cur]);   // (mu, packed) pairs
     auto hist = [&](int s) {
         const DevStack &st = a.stacks[s];
@@ -245,7 +247,7 @@ __device__ __forceinline__ void phase_wdep(const Args &a, uint32_t step)
 template <bool SM>
 __global__ void __launch_bounds__(TPB) k_wdep(const Args a)
 {
-    if (range_done(a)) phase_wdep<SM>(a, a.step_dev ? __ldcg(a.step_dev) - 1u : a.step);
+    phase_wdep<SM>(a, a.step_dev ? __ldcg(a.step_dev) - 1u : a.step);
 }
 
 // What a reading call takes to the host: a stack's counters and the device

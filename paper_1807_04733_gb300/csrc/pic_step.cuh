@@ -367,11 +367,17 @@ __device__ __forceinline__ bool timed_out(const Args &a)
 
 // Whether the grouped steps before this launch have come to the end of their
 // range (they have not after a given-up wait: the window and the state that the
-// launch is for are not there).  Uniform over the grid.
-__device__ __forceinline__ bool range_done(const Args &a)
-{
-    return !a.due || __ldcg(&a.ctl->step) == (a.due_base ? __ldcg(a.due_base) : 0u) + a.due_step;
-}
+// launch is for are not there).  Uniform over the grid.  Asked for with a launch's
+// first loads and looked at when they have come: a load of its own before them,
+// or of a graph's first step beside them, took 1 to 2 us of each launch.
+struct RangeEnd {
+    uint32_t now;
+    __device__ __forceinline__ explicit RangeEnd(const Args &a) : now(a.due ? __ldcg(&a.ctl->step) : 0u) {}
+    __device__ __forceinline__ bool reached(const Args &a) const
+    {
+        return !a.due || (a.due_period ? now >= a.due_step && (now - a.due_step) % a.due_period == 0 : now == a.due_step);
+    }
+};
 
 // Per-block plan shared by the streaming kernels: tiles of every stack
 // concatenated; this block owns tiles [t0, t1).
@@ -2167,8 +2173,10 @@ __device__ __forceinline__ void phase_compact(const Args &a)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long S = a.mp_stride;
     const unsigned int lt = (1u << lane) - 1u;
+    const RangeEnd end(a);
     for (int i = tid; i < a.n_stacks; i += TPB) s_nsl[i] = (long long)a.cnt[i].n_slots;
     cta_sync();
+    if (!end.reached(a)) return;
     // the largest tiles that give every block one
     long long all = 0;
     for (int i = 0; i < a.n_stacks; ++i) all += s_nsl[i];
@@ -2301,7 +2309,7 @@ __device__ __forceinline__ void phase_compact(const Args &a)
 template <int ADJ = 0>
 __global__ void __launch_bounds__(TPB, 4) k_compact(const Args a)
 {
-    if (range_done(a)) phase_compact<ADJ>(a);
+    phase_compact<ADJ>(a);
 }
 
 // Grid barrier: every block resident (a cooperative launch).  Sense by
