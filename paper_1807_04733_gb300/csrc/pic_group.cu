@@ -785,8 +785,8 @@ struct TailStack {                   // what a tail block keeps of its stack
     float *Z, *MU;
     uint32_t *ID, *W;
     bool vmom;
-    // births minus removals, generation and velocity sums of the group's windows
-    // (from tj0) in shared memory; null: added in memory
+    // SUMS: births minus removals, generation and velocity sums of the group's
+    // windows (from tj0) in shared memory; else added in memory
     int tj0;
     int32_t *J;
     uint32_t *G;
@@ -805,14 +805,15 @@ __host__ __device__ inline size_t tail_sums(const Args &a, int nd, int nj)
 }
 
 // the density, generation and velocity sums of one carrier at the end of window t
+template <bool SUMS>
 __device__ __forceinline__ void tail_deposit(const Args &a, const TailStack &x, int t, int sg, int k,
                                              uint32_t gen, float z, float w)
 {
     const int c = cell_at(z, a.inv_dz, x.nc);
     agg_add(&a.n_hist[x.st->n_off + ((long long)t * 2 + sg) * x.ne * x.nc + (long long)(k - 1) * x.nc + c], 1);
-    if (x.G) atomicAdd(&x.G[(t - x.tj0) * x.nc + c], gen);
+    if (SUMS) atomicAdd(&x.G[(t - x.tj0) * x.nc + c], gen);
     else agg_sum(&a.g_hist[x.st->n_off / (2 * x.ne) + (long long)t * x.nc + c], gen);
-    if (x.vmom && x.V)
+    if (SUMS && x.vmom)
         add_u64_split(&x.V[((t - x.tj0) * 2 + sg) * x.nc + c], (unsigned long long)vel_q(w));
     else if (x.vmom)
         atomicAdd(reinterpret_cast<unsigned long long *>(a.v_hist) + x.st->n_off / x.ne +
@@ -821,11 +822,12 @@ __device__ __forceinline__ void tail_deposit(const Args &a, const TailStack &x, 
 }
 
 // a birth (+1) or removal (-1) in window t, with its weight
+template <bool SUMS>
 __device__ __forceinline__ void tail_change(const Args &a, const TailStack &x, int t, int sg, float z, int by, uint32_t w)
 {
     const int c = cell_at(z, a.inv_dz, x.nc);
     const long long i = x.st->J_off + ((long long)t * 2 + sg) * x.nf + c;
-    if (x.J) atomicAdd(&x.J[((t - x.tj0) * 2 + sg) * x.nf + c], by);
+    if (SUMS) atomicAdd(&x.J[((t - x.tj0) * 2 + sg) * x.nf + c], by);
     else agg_add(reinterpret_cast<uint32_t *>(&a.bd_hist[i]), by);
     if (a.w[0])
         atomicAdd(reinterpret_cast<unsigned long long *>(a.bdw) + i,
@@ -833,6 +835,7 @@ __device__ __forceinline__ void tail_change(const Args &a, const TailStack &x, i
 }
 
 // Source(dt/2): the carrier with id `id` in slot `slot`
+template <bool SUMS>
 __device__ __forceinline__ void tail_source(const Args &a, const TailStack &x, uint32_t step, int t,
                                             unsigned long long id, long long slot, bool deposit,
                                             unsigned long long &q, unsigned long long &wsum)
@@ -877,14 +880,14 @@ __device__ __forceinline__ void tail_source(const Args &a, const TailStack &x, u
         x.W[slot] = wq;
         wsum += wq;
     }
-    tail_change(a, x, t, (int)sg, z, 1, wq);
+    tail_change<SUMS>(a, x, t, (int)sg, z, 1, wq);
     if (deposit) {
         const float v = x.vmom ? a.ent[st.ent_off + (layer * 2 + sg) * x.ne + (k - 1)].v : 0.f;
-        tail_deposit(a, x, t, (int)sg, (int)k, 1u, z, __fmul_rn(v, mu));
+        tail_deposit<SUMS>(a, x, t, (int)sg, (int)k, 1u, z, __fmul_rn(v, mu));
     }
 }
 
-template <bool DET>
+template <bool DET, bool SUMS>
 __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, const Span sp, bool no_src)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -926,12 +929,8 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
         x.W = a.w[0] ? a.w[cur] + st.base : nullptr;
         x.vmom = (a.flags & PIC_F_VELOCITY_MOMENTS) != 0;
         x.tj0 = (int)(sp.s0 / me);
-        x.J = nullptr; x.G = nullptr; x.V = nullptr;
-        // (32 bits hold the generation sums of 2^24 carriers)
-        const bool sums = g.tail_sums && st.cap / nbk < (1 << 24);
-        const int nv = sums && x.vmom && g.nd > 0 ? g.nd * 2 * x.nc : 0, nj = sums ? g.nj * 2 * x.nf : 0,
-                  ng = sums ? g.nd * x.nc : 0;
-        if (sums) {
+        const int nv = SUMS && x.vmom && g.nd > 0 ? g.nd * 2 * x.nc : 0, nj = g.nj * 2 * x.nf, ng = g.nd * x.nc;
+        if (SUMS) {
             x.V = reinterpret_cast<unsigned long long *>((reinterpret_cast<uintptr_t>(s_T + a.T_max) + 7) & ~uintptr_t(7));
             x.J = reinterpret_cast<int32_t *>(x.V + nv);
             x.G = reinterpret_cast<uint32_t *>(x.J + nj);
@@ -1070,7 +1069,7 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
                 uint2 mp = mp_next;
                 ask(xi + TPB);
                 if (slot >= nsl) {
-                    tail_source(a, x, step, t, nid + (unsigned long long)(slot - nsl), slot, false, q_src, w_src);
+                    tail_source<SUMS>(a, x, step, t, nid + (unsigned long long)(slot - nsl), slot, false, q_src, w_src);
                     z = __ldcg(x.Z + slot);
                     mp = __ldcg(reinterpret_cast<const uint2 *>(x.MU + 2 * slot));
                 }
@@ -1123,7 +1122,7 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
                         }
                         if (dead) {
                             pk = (pk & ~0x1FFFu) | ((uint32_t)sg << 8) | ((uint32_t)layer << 9);
-                            tail_change(a, x, t, sg, z, -1, a.w[0] ? x.W[slot] : 0u);
+                            tail_change<SUMS>(a, x, t, sg, z, -1, a.w[0] ? x.W[slot] : 0u);
                             atomicAdd(&g.abs[s * GROUP_MAX + j], 1u);
                         } else {
                             flight<DET>(a, S, z, mu, layer, e, lo, hi, sg, k, half, (uint32_t)slot, x.ctr_hi,
@@ -1137,7 +1136,7 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
                         }
                     }
                     x.Z[slot] = z;
-                    if (dep && !dead) tail_deposit(a, x, t, sg, k, (pk >> 13) & 0xFFu, z, w_end);
+                    if (dep && !dead) tail_deposit<SUMS>(a, x, t, sg, k, (pk >> 13) & 0xFFu, z, w_end);
                 }
                 list[slot] = rec;
             }
@@ -1199,8 +1198,8 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
                     wp = __ldcg(&x.W[c.pslot]);
                     x.W[d] = wp;
                 }
-                tail_change(a, x, t, sg, c.zb, 1, wp);
-                if (dep) tail_deposit(a, x, t, sg, ks, (c.pk >> 13) & 0xFFu, c.z, __fmul_rn(c.v, c.mu));
+                tail_change<SUMS>(a, x, t, sg, c.zb, 1, wp);
+                if (dep) tail_deposit<SUMS>(a, x, t, sg, ks, (c.pk >> 13) & 0xFFu, c.z, __fmul_rn(c.v, c.mu));
             };
             if (s_tot[j] > 0) {
                 // a thread per record, in pieces of the block's sub-tiles
@@ -1237,7 +1236,7 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
             const long long r1 = st.cap - nsl;
             const long long i1 = in1 < r1 ? in1 : (r1 > 0 ? r1 : 0);
             for (long long xi = (long long)ib * TPB + tid; xi < i1; xi += (long long)nbk * TPB)
-                tail_source(a, x, step, t, nid + (unsigned long long)xi, nsl + xi, dep, q_src, w_src);
+                tail_source<SUMS>(a, x, step, t, nid + (unsigned long long)xi, nsl + xi, dep, q_src, w_src);
             if (ib == 0 && tid == 0) {
                 unsigned long long *led = a.cnt[s].led;
                 if (i1) atomicAdd(&led[L_INJECTED], (unsigned long long)i1);
@@ -1256,7 +1255,7 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
             }
         }
         // ---- the block's sums and counts
-        if (sums) {
+        if (SUMS) {
             cta_sync();
             int32_t *gJ = a.bd_hist + st.J_off + (long long)x.tj0 * 2 * x.nf;
             unsigned long long *gG = a.g_hist + st.n_off / (2 * x.ne) + (long long)x.tj0 * x.nc;
@@ -1313,13 +1312,13 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
     }
 }
 
-template <bool DET>
+template <bool DET, bool SUMS>
 __global__ void __launch_bounds__(TPB, 2) k_tail(const Args a, const GroupArgs g)
 {
     const uint32_t s0 = (g.base ? __ldcg(g.base) : 0u) + (uint32_t)g.off;
     const Span sp = g.nd > 0 ? group_span<true>(a, s0, g.end - g.off, g.m, g.no_src != 0)
                              : group_span<false>(a, s0, g.end - g.off, g.m, g.no_src != 0);
-    if (sp.len != 0) phase_tail<DET>(a, g, sp, g.no_src != 0);
+    if (sp.len != 0) phase_tail<DET, SUMS>(a, g, sp, g.no_src != 0);
 }
 
 // ---------------------------------------------------------------------------
@@ -1345,8 +1344,8 @@ __device__ __forceinline__ void phase_dens(const Args &a)
     long long *s_nsl = s_tpref + a.n_stacks + 1;
     const int tid = threadIdx.x, ne = a.n_e;
     const int cur = (int)__ldcg(&a.ctl->cur);
-    const RangeEnd end(a);
     const int t = (int)(__ldcg(&a.ctl->step) / (uint32_t)a.moment_every) - 1;
+    const RangeEnd end(a);
     for (int s = tid; s < a.n_stacks; s += NT) s_nsl[s] = (long long)a.cnt[s].n_slots;
     __syncthreads();
     if (tid == 0) {
@@ -1451,7 +1450,8 @@ __global__ void __launch_bounds__(32 * GW_MAX, 1) k_run(const Args a, const Grou
             if (sp.len == 0) return;         // (only after a wait was given up in k_tail's part)
             phase_group<DET, DEP, Q>(a, g, sp);
             if (!grid_sync(a)) return;
-            if (low) phase_tail<DET>(a, g, sp, no_src);
+            if (low && g.tail_sums) phase_tail<DET, true>(a, g, sp, no_src);
+            else if (low) phase_tail<DET, false>(a, g, sp, no_src);
             if (!grid_sync(a)) return;
             s += (uint32_t)sp.len;
         }
@@ -1563,12 +1563,15 @@ cudaError_t configure_group(const Args &a, long long slots, GroupCfg *gc)
     }
     if (!c.ok) return cudaSuccess;
     c.smem_tail = (size_t)a.tab_max * sizeof(TabEnt) + (size_t)a.T_max * 4 + 16;
-    // (two blocks per SM keep theirs beside the tables)
-    c.tail_sums = tail_sums(a, c.nd, c.nj) <= 48 * 1024;
+    // Two blocks per SM keep theirs beside the tables.  Births and removals alone
+    // are too few in small contexts to pay for clearing and flushing (300 steps
+    // from 1e5 carriers 4.56 ms without, 4.67 with).
+    c.tail_sums = (c.dep || slots > (1ll << 20)) && tail_sums(a, c.nd, c.nj) <= 48 * 1024;
     if (c.tail_sums) c.smem_tail += tail_sums(a, c.nd, c.nj);
     int o1 = 0, o2 = 0;
-    e = occupancy(k_tail<false>, c.smem_tail, &o1);
-    if (e == cudaSuccess) e = occupancy(k_tail<true>, c.smem_tail, &o2);
+    e = c.tail_sums ? occupancy(k_tail<false, true>, c.smem_tail, &o1) : occupancy(k_tail<false, false>, c.smem_tail, &o1);
+    if (e == cudaSuccess)
+        e = c.tail_sums ? occupancy(k_tail<true, true>, c.smem_tail, &o2) : occupancy(k_tail<true, false>, c.smem_tail, &o2);
     if (e != cudaSuccess) return e;
     const int ot = std::min({o1, o2, 2});
     if (ot < 1 || sms * ot < a.n_stacks) return cudaSuccess;
@@ -1683,7 +1686,9 @@ cudaError_t launch_tail(const Args &a, const GroupArgs &g, const GroupCfg &c, bo
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return det ? cudaLaunchKernelEx(&cfg, k_tail<true>, a, g) : cudaLaunchKernelEx(&cfg, k_tail<false>, a, g);
+    if (g.tail_sums)
+        return det ? cudaLaunchKernelEx(&cfg, k_tail<true, true>, a, g) : cudaLaunchKernelEx(&cfg, k_tail<false, true>, a, g);
+    return det ? cudaLaunchKernelEx(&cfg, k_tail<true, false>, a, g) : cudaLaunchKernelEx(&cfg, k_tail<false, false>, a, g);
 }
 
 cudaError_t launch_dens(const Args &a, const GroupCfg &c, cudaStream_t s)
