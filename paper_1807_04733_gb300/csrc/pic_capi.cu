@@ -1097,6 +1097,16 @@ int range_end(const pic_ctx *c, int s)
     return e;
 }
 
+// Whether a step by itself, the one before time step s1 (counted from a multiple
+// of the period in graphs), takes the single-step kernels (LONE_SLOTS).
+bool lone_single(const pic_ctx *c, int s1, bool src)
+{
+    if (src) return false;
+    if (s1 % c->p.moment_every == 0)
+        return c->total_slots > ((c->p.flags & PIC_F_WEIGHTS) ? LONE_SLOTS_WEIGHTS : LONE_SLOTS);
+    return c->total_slots > LONE_SLOTS && c->total_slots <= LONE_SLOTS_MOST;
+}
+
 // Steps [s, e) in groups, then what is due at their end.  Every group's
 // launches are issued for the case that the groups before it were open; one
 // that a closed group has run past leaves at once.  `base`: s and e count from
@@ -1187,7 +1197,8 @@ cudaError_t capture_period(pic_ctx *c, int which)
         ++n;
         for (int i = 0; i < c->period && e == cudaSuccess;) {
             const int i1 = std::min(range_end(c, i), c->period);
-            e = enqueue_range(c, a, i, i1, &c->d_ctl->base, src, c->cap_stream, n);
+            if (i1 - i == 1 && lone_single(c, i1, src)) e = enqueue_step(c, a, i, false, false, true, c->cap_stream, n);
+            else e = enqueue_range(c, a, i, i1, &c->d_ctl->base, src, c->cap_stream, n);
             i = i1;
         }
     } else {
@@ -1339,9 +1350,9 @@ pic_status pic_step(pic_ctx *c, int n_steps)
             left -= c->period;
             continue;
         }
-        if (grouped(c)) {
-            const bool run = run_plain(c) && left > c->gc.m;
-            const int s1 = run ? s + left : std::min(range_end(c, s), s + left);
+        const bool run = grouped(c) && run_plain(c) && left > c->gc.m;
+        const int s1 = run ? s + left : std::min(range_end(c, s), s + left);
+        if (grouped(c) && (s1 - s > 1 || !lone_single(c, s1, any_source(c, s, 1)))) {
             if (!c->dev_step_valid) {
                 e = launch_set_step(c->d_ctl, (unsigned int)s, c->stream);
                 c->launches += 1;

@@ -1516,6 +1516,10 @@ std::vector<GroupShape> group_shapes(const Args &a, long long slots, int sms, si
     for (int m = slots <= GROUP_LIST_SLOTS ? GROUP_OPEN : GROUP_OPEN_LARGE; m >= 1; --m) {
         const int nd = dep ? (me - 1 + m) / me : 0;
         const int nj = dep ? (me + m - 2) / me + 1 : 1;
+        // groups of one step (50 steps of 245 cells x 60 bins: 1.2e6 slots 1.57 ms, single
+        // steps 2.02; 1.2e7 slots 6.43 and 5.44; densities every third step, 275
+        // cells: 1.69 and 1.63)
+        if (m == 1 && (me > 1 || slots > LONE_SLOTS)) break;
         // too few warps beside the histograms: fewer windows
         const int least = m == 1 || quads == 8 ? TPB / 32 : quads == 4 ? (m > GROUP_OPEN_LARGE ? 14 : TPB / 32) : 12;
         for (int w = GW_MAX; w >= least; --w) {

@@ -222,6 +222,17 @@ struct Args {            // everything a kernel needs, passed by value
 // lists of more steps would need memory of their own.
 constexpr int GROUP_OPEN = 8, GROUP_OPEN_LARGE = 4;
 constexpr long long GROUP_LIST_SLOTS = 8ll << 20;
+// A step by itself (a call of one step, or densities so often and of so many bins
+// that a group holds one window) saves no pass over memory; the single-step
+// kernels have more warps and less fixed work per carrier, and two launches more.
+// Ten calls of one step, single and in groups: with densities 0.408 and 0.397 ms at
+// 2e6 slots, 0.432 and 0.465 at 3e6, 2.37 and 3.31 at 4e7; without 0.346 and 0.388
+// at 3e6, 0.92 and 1.08 at 1.6e7, but 19.0 and 17.4 at 4e8.  With weights, whose
+// densities are passes of their own, 0.48 and 0.51 at 1e6, 4.4 and 5.9 at 4e7, but
+// 6.6 and 5.9 for 150 steps of 8e4 slots.  Steps with a source stay groups, which
+// take its carriers along (140 steps of a pulse of 1e6 weighted carriers,
+// densities every step: 10.2 ms, single steps 12.5).
+constexpr long long LONE_SLOTS = 2ll << 20, LONE_SLOTS_WEIGHTS = 1ll << 19, LONE_SLOTS_MOST = 128ll << 20;
 constexpr int GROUP_DEP_EVERY = 4;   // densities inside the groups if taken more often than this
 constexpr int GROUP_MAX = 64;    // most steps of a closed group
 constexpr int GROUP_SUB_MIN = 256;   // fewest slots of a warp's sub-tile

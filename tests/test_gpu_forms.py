@@ -23,3 +23,14 @@ def test_large_density_grid(cells, me):
     wl = W.bilayer(fe_nm=15, au_nm=cells - 15, n0=300_000, capacity=1_200_000, n_e=60,
                    n_steps=130, moment_every=me, flags=DET)
     assert check(wl, [101, 1, 28])[3]["eventful"] > 0
+
+
+@pytest.mark.parametrize("flags", [0, W.FLAG_WEIGHTS, W.FLAG_VELOCITY])
+@pytest.mark.parametrize("me", [1, 4])
+def test_calls_of_one_step_between_others(me, flags):
+    """More slots than LONE_SLOTS: a step by itself takes the single-step kernels,
+    and the groups before and after it go on from its state."""
+    wl = W.bilayer(n0=300_000, capacity=2_500_000, n_steps=160, moment_every=me, flags=DET | flags)
+    led = check(wl, [95, 1, 1, 3, 1, 20, 1, 1, 1, 36])[3]
+    assert led["injected"] > 0 and led["spawned"] > 0
+    check(wl, [101, 1, 58], graph=1)
