@@ -27,7 +27,8 @@ constexpr int TPB = 256;            // threads per block of the streaming kernel
 constexpr int VEC = 4;              // particles per thread per tile (128-bit)
 constexpr int TILE = TPB * VEC;     // particles per tile
 constexpr int LEDGER_N = 14;        // fields of pic_ledger
-constexpr int COMPACT_TILE = 16384; // most slots per tile of the compaction
+constexpr int COMPACT_TILE = 16384; // most slots per tile of the compaction, and fewest
+constexpr int COMPACT_TILE_MIN = 8 * TPB;
 // look-back words of the compaction of n slots in S stacks by a grid of G blocks
 // (tiles are smaller where the largest would leave blocks without one)
 constexpr long long compact_words(long long n, int G, int S)

@@ -16,6 +16,7 @@
 // on the GPU (different streams, or host threads) race on it.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -132,7 +133,9 @@ extern "C" pic_status pic_compact_static(const float *z, const float *mu, const 
     a.ctl = &scr->ctl;
     a.spin_limit = 1u << 24;
     LaunchCfg c{};
-    c.grid_compact = grid;
+    // no more blocks than tiles: each takes a ticket and reports its end (one call
+    // on 1e3 slots 56 us with 608 blocks, 45 with one)
+    c.grid_compact = (int)std::min<int64_t>(grid, (n + COMPACT_TILE_MIN - 1) / COMPACT_TILE_MIN);
     e = launch_compact(a, c, stream);
     if (e != cudaSuccess) return cuda_error(e, "pic_compact_static: launch");
 

@@ -2167,7 +2167,8 @@ __device__ __forceinline__ void phase_compact(const Args &a)
     __shared__ long long s_prefix;
     __shared__ int s_flag;
     constexpr int CV = 8;                                    // rows at a time
-    constexpr int CS = TPB * CV;                             // smallest tile
+    constexpr int CS = COMPACT_TILE_MIN;
+    static_assert(CS == TPB * CV, "a tile of one group of rows per warp");
     const unsigned int ep = *(volatile unsigned int *)&a.ctl->epoch;
     const int cur = (int)*(volatile unsigned int *)&a.ctl->cur, nxt = cur ^ 1;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
