@@ -838,7 +838,6 @@ pic_status pic_init(pic_ctx **out, const pic_params *p, const pic_stack_desc *st
         if (e == cudaSuccess) e = dalloc(&c->d_gbar, (size_t)32 * n_stacks);
         if (e == cudaSuccess) e = dalloc(&c->d_gblk, gt + gr);
         // every stack one block, the others by capacity (the rest to the largest)
-        int64_t most = 0;                        // slots per block of a stack
         auto share = [&](int total) {
             std::vector<int> nb(n_stacks, 1);
             int left = total - n_stacks, big = 0;
@@ -853,16 +852,12 @@ pic_status pic_init(pic_ctx **out, const pic_params *p, const pic_stack_desc *st
             nb[big] += left;
             int first = 0;
             for (int s = 0; s < n_stacks; ++s) {
-                most = std::max(most, c->hs[s].cap_round / nb[s]);
                 for (int i = 0; i < nb[s]; ++i) blk.push_back(make_int4(s, i, nb[s], first));
                 first += nb[s];
             }
         };
         share(gt);
         if (c->gc.run) share(gr);
-        // (32 bits hold the generation sums of the carriers of 2^22 slots: those a
-        // block moves, those it places and those of the source, 255 each)
-        if (most > (1ll << 22)) c->gc.tail_sums = false;
         // the lists of the steps: one 8-byte record per slot and step, in the
         // buffers of the single steps' staged and queued records, and more for
         // groups of more than four steps

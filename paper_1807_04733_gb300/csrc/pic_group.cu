@@ -1566,22 +1566,30 @@ cudaError_t configure_group(const Args &a, long long slots, GroupCfg *gc)
         break;
     }
     if (!c.ok) return cudaSuccess;
-    c.smem_tail = (size_t)a.tab_max * sizeof(TabEnt) + (size_t)a.T_max * 4 + 16;
-    // Two blocks per SM keep theirs beside the tables.  Births and removals alone
-    // are too few in small contexts to pay for clearing and flushing (300 steps
-    // from 1e5 carriers 4.56 ms without, 4.67 with).
-    c.tail_sums = (c.dep || slots > (1ll << 20)) && tail_sums(a, c.nd, c.nj) <= 48 * 1024;
-    if (c.tail_sums) c.smem_tail += tail_sums(a, c.nd, c.nj);
-    int o1 = 0, o2 = 0;
-    e = c.tail_sums ? occupancy(k_tail<false, true>, c.smem_tail, &o1) : occupancy(k_tail<false, false>, c.smem_tail, &o1);
-    if (e == cudaSuccess)
-        e = c.tail_sums ? occupancy(k_tail<true, true>, c.smem_tail, &o2) : occupancy(k_tail<true, false>, c.smem_tail, &o2);
+    // Blocks: every one resident (they wait on one another), few for few carriers.
+    // Two per SM keep their sums over cells beside the tables.  Births and removals
+    // alone are too few in small contexts to pay for clearing and flushing (300
+    // steps from 1e5 carriers 4.56 ms without, 4.67 with), and 32 bits hold the
+    // generation sums of the carriers that a block moves and of those that it
+    // places, each at most its stack's share (pic_init) of 2^23 slots, 255 each.
+    auto tail = [&](bool sums) -> cudaError_t {
+        c.tail_sums = sums;
+        c.smem_tail = (size_t)a.tab_max * sizeof(TabEnt) + (size_t)a.T_max * 4 + 16 + (sums ? tail_sums(a, c.nd, c.nj) : 0);
+        int o1 = 0, o2 = 0;
+        cudaError_t r = sums ? occupancy(k_tail<false, true>, c.smem_tail, &o1) : occupancy(k_tail<false, false>, c.smem_tail, &o1);
+        if (r == cudaSuccess)
+            r = sums ? occupancy(k_tail<true, true>, c.smem_tail, &o2) : occupancy(k_tail<true, false>, c.smem_tail, &o2);
+        const long long most = (long long)sms * std::min({o1, o2, 2});
+        c.grid_tail = (int)std::max<long long>(std::min<long long>(std::max<long long>(slots / 4096, 8), most), a.n_stacks);
+        if (most < a.n_stacks) c.grid_tail = 0;
+        return r;
+    };
+    e = tail((c.dep || slots > (1ll << 20)) && tail_sums(a, c.nd, c.nj) <= 48 * 1024);
+    if (e == cudaSuccess && c.tail_sums &&
+        slots / std::max(std::min(c.grid_tail, c.grid) - a.n_stacks, 1) > (1ll << 23))
+        e = tail(false);
     if (e != cudaSuccess) return e;
-    const int ot = std::min({o1, o2, 2});
-    if (ot < 1 || sms * ot < a.n_stacks) return cudaSuccess;
-    // every block resident (they wait on one another); few for few carriers
-    long long gt = std::max<long long>(slots / 4096, 8);
-    c.grid_tail = (int)std::max<long long>(std::min<long long>(gt, (long long)sms * ot), a.n_stacks);
+    if (c.grid_tail == 0) return cudaSuccess;
     if (!c.dep) {
         c.smem_dens = dens_smem(a);
         int od = 0;

@@ -34,3 +34,11 @@ def test_calls_of_one_step_between_others(me, flags):
     led = check(wl, [95, 1, 1, 3, 1, 20, 1, 1, 1, 36])[3]
     assert led["injected"] > 0 and led["spawned"] > 0
     check(wl, [101, 1, 58], graph=1)
+
+
+def test_many_stacks_and_a_large_one():
+    """One block for a stack of more slots than 32-bit sums are safe for."""
+    wl = W.batched(n_stacks=151, scale=2e-4, n_steps=120, flags=DET)
+    wl.stacks[3].capacity = 9_000_000
+    led = check(wl, [100, 20])[3]
+    assert led["injected"] > 0
