@@ -2177,17 +2177,19 @@ pic_status pic_autotune(pic_ctx *c, int trial_steps, pic_tune_entry *entries, in
     // the fused form exists for one stack and eight consumer warps, with at
     // most PIC_EV_MIN_BLOCKS blocks per SM
     const bool fusable = c->n_stacks == 1;
-    // grouped steps do not depend on the other options: one ring depth and
-    // deposit mode of them are tried
+    // Grouped steps do not depend on the other options: they are one candidate, with
+    // the most blocks and the deepest ring that fit for the steps between groups;
+    // the last, as a run whose carriers still grow favours later trials (tried
+    // first, with a source, they were taken for slower where they take a third).
     const bool grp = c->gc.ok;
     for (int hm = 0; hm <= (dep_in_trial ? 1 : 0); ++hm)
         for (int nw : {8, 4})
-            for (int ev = (nw == 8 && (fusable || grp) ? 0 : 1); ev <= 1; ++ev)
+            for (int ev = (nw == 8 && fusable && !grp ? 0 : 1); ev <= 1; ++ev)
                 for (int bps = 1; bps <= (ev == 0 ? 3 : nw == 4 ? 8 : 6); ++bps)
-                    for (int ring : {2, 3, 4, 6, 8}) {
-                        if (ev == 0 && grp && (ring != 2 || hm != 0)) continue;
-                        cands.push_back({bps, ring, hm, nw, ev});
-                    }
+                    for (int ring : {2, 3, 4, 6, 8}) cands.push_back({bps, ring, hm, nw, ev});
+    if (grp)
+        for (int bps : {3, 2, 1})
+            for (int ring : {8, 6, 4, 3, 2}) cands.push_back({bps, ring, 0, 8, 0});
     // a trial of grouped steps has at least a whole group (with two steps where a
     // group has four the spin valve's were taken for slower than single ones);
     // the budget of steps is that of single ones, one trial per configuration
@@ -2222,6 +2224,7 @@ pic_status pic_autotune(pic_ctx *c, int trial_steps, pic_tune_entry *entries, in
     std::vector<pic_tune_entry> res;
     for (size_t i = 0; i < cands.size() && e == cudaSuccess; ++i) {
         const Cand &k = cands[i];
+        if (k.ev == 0 && grp && !res.empty() && res.back().event_pass == 0) continue;
         if ((int64_t)(c->step - first_step) + steps_of(k) > budget) continue;
         LaunchCfg lc{};
         if (configure(c->args, k.bps, k.ring, k.hm, k.nw, &lc) != cudaSuccess) {
@@ -2232,12 +2235,13 @@ pic_status pic_autotune(pic_ctx *c, int trial_steps, pic_tune_entry *entries, in
                                    lc.grid_slow_dep, lc.grid_place, lc.grid_place_dep,
                                    lc.grid_compact});
         // a candidate whose ring leaves fewer resident blocks than asked for
-        // is another candidate's duplicate
+        // is another candidate's duplicate (the fused form's shape does not matter
+        // to grouped steps)
         if (k.ev == 1) lc.grid_fused = 0;
         if (gmax > c->n_status || lc.ring_fast != k.ring || lc.grid_fast != sms * k.bps ||
             lc.grid_fast_dep == 0)
             continue;
-        if (k.ev == 0 && fusable && (lc.grid_fused != sms * k.bps || lc.ring_fused != k.ring)) continue;
+        if (k.ev == 0 && !grp && (lc.grid_fused != sms * k.bps || lc.ring_fused != k.ring)) continue;
         c->lc = lc;
         c->p.hist_mode = k.hm;
         c->p.event_pass = k.ev;

@@ -42,3 +42,20 @@ def test_many_stacks_and_a_large_one():
     wl.stacks[3].capacity = 9_000_000
     led = check(wl, [100, 20])[3]
     assert led["injected"] > 0
+
+
+@pytest.mark.parametrize("stacks", [1, 3])
+def test_autotune_tries_grouped_steps_once(stacks):
+    """One trial of grouped steps, also beside the little that 16 layers of 100 bins
+    leave of the fused form, and for several stacks."""
+    if stacks == 1:
+        st = W.make_stack([5] * 16, [i % 3 for i in range(16)], 100, 0.02, 30_000, 10_000)
+        wl = W.Workload("layers", 100, 0.02, 1.0, 1.0, 900, 50, 50, 3, DET, [st])
+    else:
+        wl = W.batched(n_stacks=3, scale=1e-3, n_steps=900, moment_every=50, flags=DET)
+    ctx = pic.Context(wl)
+    ctx.step(100)
+    trials = ctx.autotune(3)
+    assert sum(t["event_pass"] == 0 for t in trials) == 1
+    assert sum(t["chosen"] for t in trials) == 1
+    ctx.close()
