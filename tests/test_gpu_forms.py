@@ -59,3 +59,43 @@ def test_autotune_tries_grouped_steps_once(stacks):
     assert sum(t["event_pass"] == 0 for t in trials) == 1
     assert sum(t["chosen"] for t in trials) == 1
     ctx.close()
+
+
+def single(wl):
+    """The workload with one certain scattering (the lowest bin of one table):
+    thresholds that close to 1 keep its steps from being grouped."""
+    wl.stacks[0].tau_in = wl.stacks[0].tau_in.copy()
+    wl.stacks[0].tau_in[1, 1, 0] = 1e-9
+    return wl
+
+
+@pytest.mark.parametrize("graph", [0, 1, 2])
+@pytest.mark.parametrize("me,flags", [(1, 0), (50, 0), (5, W.FLAG_VELOCITY), (5, W.FLAG_WEIGHTS)])
+def test_single_steps(me, flags, graph):
+    """Steps that are not grouped: the general step inside the streaming pass
+    (fused), graphs of single steps and the persistent kernel of their passes."""
+    wl = single(W.bilayer(n0=20_000, capacity=50_000, n_steps=250, moment_every=me, flags=DET | flags))
+    ctx = pic.Context(wl)
+    ctx.step(10)
+    assert ctx.launches >= 20                      # a launch per pass and step
+    ctx.close()
+    assert check(wl, [50, 130, 70], graph=graph)[3]["spawn_dropped"] > 0
+
+
+@pytest.mark.parametrize("graph", [0, 2])
+@pytest.mark.parametrize("me,chunks", [(1, [60, 40, 100]), (5, [200]), (50, [75, 125])])
+def test_persistent_groups(me, chunks, graph):
+    wl = W.spin_valve(True, fe_nm=5, au_nm=30, n0=20_000, capacity=60_000, n_steps=200, moment_every=me,
+                      flags=DET | W.FLAG_VELOCITY)
+    check(wl, chunks, graph=graph)
+
+
+@pytest.mark.parametrize("graph", [0, 1, 2])
+@pytest.mark.parametrize("capacity,n", [(3_000_000, 3_000_000), (9_000_000, 8_990_000)])
+def test_closed_groups_of_large_sub_tiles(capacity, n, graph):
+    """1024-slot sub-tiles and groups of up to 50 steps: a full buffer, and one
+    that fills up in the first steps, above the size of the plain persistent form
+    (several launches per range, of which a closed group's successors leave)."""
+    wl = W.bilayer(n0=0, capacity=capacity, n_steps=170, moment_every=50, flags=DET)
+    led = check(wl, [20, 100, 50], records(wl, n), graph=graph)[3]
+    assert led["spawn_dropped"] > 0 and led["absorbed"] > 0
