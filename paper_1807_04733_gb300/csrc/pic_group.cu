@@ -1550,8 +1550,7 @@ cudaError_t configure_group(const Args &a, long long slots, GroupCfg *gc)
     for (const GroupShape &x : group_shapes(a, slots, sms, cap)) {
         bool ok = false;
         if (c.dep) {
-            if (x.quads == 8) e = group_fits<true, 8>(x.smem, 32 * x.warps, &ok);
-            else if (x.quads == 4) e = group_fits<true, 4>(x.smem, 32 * x.warps, &ok);
+            if (x.quads == 4) e = group_fits<true, 4>(x.smem, 32 * x.warps, &ok);
             else e = group_fits<true, 2>(x.smem, 32 * x.warps, &ok);
         } else {
             if (x.quads == 8) e = group_fits<false, 8>(x.smem, 32 * x.warps, &ok);
@@ -1625,8 +1624,7 @@ static cudaError_t configure_run(const Args &a, GroupCfg *c)
         c->smem_run = std::max({group_smem(a, c->dep, c->quads, w, c->nd, c->nj).total, c->smem_tail, c->smem_dens});
         c->warps_run = w;
         if (c->dep) {
-            if (c->quads == 8) e = run_fits<true, 8>(c->smem_run, 32 * w, &c->run);
-            else if (c->quads == 4) e = run_fits<true, 4>(c->smem_run, 32 * w, &c->run);
+            if (c->quads == 4) e = run_fits<true, 4>(c->smem_run, 32 * w, &c->run);
             else e = run_fits<true, 2>(c->smem_run, 32 * w, &c->run);
         } else {
             if (c->quads == 8) e = run_fits<false, 8>(c->smem_run, 32 * w, &c->run);
@@ -1654,7 +1652,6 @@ cudaError_t launch_run(const Args &a, const GroupArgs &g, const GroupCfg &c, boo
     return det ? cudaLaunchKernelEx(&cfg, k_run<true, DEP, Q>, a, g, n_steps, src_end)             \
                : cudaLaunchKernelEx(&cfg, k_run<false, DEP, Q>, a, g, n_steps, src_end)
     if (c.dep) {
-        if (c.quads == 8) PIC_RUN_LAUNCH(true, 8);
         if (c.quads == 4) PIC_RUN_LAUNCH(true, 4);
         PIC_RUN_LAUNCH(true, 2);
     }
@@ -1674,8 +1671,7 @@ cudaError_t launch_group(const Args &a, const GroupArgs &g, const GroupCfg &c, b
         else k_group<false, DEP, Q><<<c.grid, nt, c.smem, s>>>(a, g);                              \
     } while (0)
     if (c.dep) {
-        if (c.quads == 8) PIC_GROUP_LAUNCH(true, 8);
-        else if (c.quads == 4) PIC_GROUP_LAUNCH(true, 4);
+        if (c.quads == 4) PIC_GROUP_LAUNCH(true, 4);
         else PIC_GROUP_LAUNCH(true, 2);
     } else {
         if (c.quads == 8) PIC_GROUP_LAUNCH(false, 8);

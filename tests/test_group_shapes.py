@@ -38,6 +38,8 @@ def test_every_shape_has_the_threads_of_its_barriers(shapes, n_stacks, layers, f
             seen += 1
             assert 8 <= warps <= 16 and quads in (2, 4, 8) and 1 <= m <= 8, (n_e, cells, me, slots)
             assert m <= 4 or slots <= 8 << 20
+            # no kernel of 1024-slot sub-tiles with densities
+            assert quads <= 4 or me >= 4 or flags & W.FLAG_WEIGHTS
             # groups of one step: densities every step and few slots
             assert m > 1 or (me == 1 and slots <= 2 << 20)
     assert seen > 1000
