@@ -887,20 +887,42 @@ __device__ __forceinline__ void tail_source(const Args &a, const TailStack &x, u
     }
 }
 
+// The static shared memory of phase_tail, one for both of its forms in k_run (with
+// two of them it had room for fewer warps: 100 steps of 4e5 slots 0.83 -> 0.98 ms).
+struct TailShared {
+    DevStack st;
+    float edge[PIC_MAX_LAYERS + 1];
+    uint32_t p0[PIC_MAX_LAYERS];
+    uint32_t pre[TAIL_PIECE + 1];
+    uint32_t tot[GROUP_OPEN], mine[GROUP_OPEN];
+    uint32_t tt[2];
+    int w[TPB / 32], flag;
+    unsigned long long r8[(TPB / 32) * 10];
+};
+
+__device__ __forceinline__ TailShared &tail_shared()
+{
+    __shared__ TailShared sh;
+    return sh;
+}
+
 template <bool DET, bool SUMS>
 __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, const Span sp, bool no_src)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     TabEnt *s_ent = reinterpret_cast<TabEnt *>(smem);
     uint32_t *s_T = reinterpret_cast<uint32_t *>(s_ent + a.tab_max);
-    __shared__ DevStack s_st;
-    __shared__ float s_edge[PIC_MAX_LAYERS + 1];
-    __shared__ uint32_t s_p0[PIC_MAX_LAYERS];
-    __shared__ uint32_t s_pre[TAIL_PIECE + 1];
-    __shared__ uint32_t s_tot[GROUP_OPEN], s_mine[GROUP_OPEN];
-    __shared__ uint32_t s_tt[2];
-    __shared__ int s_w[TPB / 32], s_flag;
-    __shared__ unsigned long long s_r8[(TPB / 32) * 10];
+    TailShared &sh = tail_shared();
+    DevStack &s_st = sh.st;
+    auto &s_edge = sh.edge;
+    auto &s_p0 = sh.p0;
+    auto &s_pre = sh.pre;
+    auto &s_tot = sh.tot;
+    auto &s_mine = sh.mine;
+    auto &s_tt = sh.tt;
+    auto &s_w = sh.w;
+    int &s_flag = sh.flag;
+    auto &s_r8 = sh.r8;
 
     const int tid = threadIdx.x, lane = tid & 31;
     const int4 bl = g.blk[blockIdx.x];
