@@ -435,8 +435,10 @@ cudaError_t configure(const Args &a, int blocks_per_sm, int ring_req, int hist_m
     cfg->grid_compact = sms * (oc > 0 ? oc : 1);
     cfg->grid_inject = sms * 4;
     // The weighted densities: the blocks that are resident beside their
-    // histograms.  (3 per SM for 115 cells of 30 bins: 26 us for 4e6 slots, 204
-    // for 4e7; with the compaction's grid, 4 per SM, 34 and 296.)
+    // histograms, at most four per SM, each of which adds its histogram to the
+    // one in memory.  (115 cells of 30 bins, 3 per SM: 38 us for 6e6 slots, 204 for
+    // 4e7; a fourth that is not resident: 34 and 296 at 4e6 and 4e7.  70 cells, 6
+    // resident: 18 us for 1.5e6 slots with 4, 22 with 6; 157 both for 4e7.)
     cfg->grid_wdep = 0;
     cfg->smem_wdep = 0;
     if (a.w[0]) {
@@ -447,7 +449,7 @@ cudaError_t configure(const Args &a, int blocks_per_sm, int ring_req, int hist_m
             cfg->smem_wdep = 0;
             if ((e = occupancy(k_wdep<false>, 0, &ow)) != cudaSuccess) return e;
         }
-        cfg->grid_wdep = sms * std::max(ow, 1);
+        cfg->grid_wdep = sms * std::max(std::min(ow, 4), 1);
     }
     return cudaSuccess;
 }
