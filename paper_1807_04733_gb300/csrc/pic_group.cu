@@ -951,7 +951,9 @@ __device__ __forceinline__ void phase_tail(const Args &a, const GroupArgs &g, co
         x.W = a.w[0] ? a.w[cur] + st.base : nullptr;
         x.vmom = (a.flags & PIC_F_VELOCITY_MOMENTS) != 0;
         x.tj0 = (int)(sp.s0 / me);
-        const int nv = SUMS && x.vmom && g.nd > 0 ? g.nd * 2 * x.nc : 0, nj = g.nj * 2 * x.nf, ng = g.nd * x.nc;
+        // the windows that the group's steps lie in, and of these the ones that may end
+        const int wj = (int)((sp.s0 + (uint32_t)sp.len - 1u) / me) - x.tj0 + 1, wd = wj < g.nd ? wj : g.nd;
+        const int nv = x.vmom ? wd * 2 * x.nc : 0, nj = wj * 2 * x.nf, ng = wd * x.nc;
         if (SUMS) {
             x.V = reinterpret_cast<unsigned long long *>((reinterpret_cast<uintptr_t>(s_T + a.T_max) + 7) & ~uintptr_t(7));
             x.J = reinterpret_cast<int32_t *>(x.V + nv);
@@ -1596,11 +1598,12 @@ cudaError_t configure_group(const Args &a, long long slots, GroupCfg *gc)
     auto tail = [&](bool sums) -> cudaError_t {
         c.tail_sums = sums;
         c.smem_tail = (size_t)a.tab_max * sizeof(TabEnt) + (size_t)a.T_max * 4 + 16 + (sums ? tail_sums(a, c.nd, c.nj) : 0);
-        int o1 = 0, o2 = 0;
-        cudaError_t r = sums ? occupancy(k_tail<false, true>, c.smem_tail, &o1) : occupancy(k_tail<false, false>, c.smem_tail, &o1);
-        if (r == cudaSuccess)
-            r = sums ? occupancy(k_tail<true, true>, c.smem_tail, &o2) : occupancy(k_tail<true, false>, c.smem_tail, &o2);
-        const long long most = (long long)sms * std::min({o1, o2, 2});
+        int o[4] = {2, 2, 2, 2};                 // (a step by itself takes the form without sums)
+        cudaError_t r = occupancy(k_tail<false, false>, c.smem_tail, &o[0]);
+        if (r == cudaSuccess) r = occupancy(k_tail<true, false>, c.smem_tail, &o[1]);
+        if (sums && r == cudaSuccess) r = occupancy(k_tail<false, true>, c.smem_tail, &o[2]);
+        if (sums && r == cudaSuccess) r = occupancy(k_tail<true, true>, c.smem_tail, &o[3]);
+        const long long most = (long long)sms * std::min({o[0], o[1], o[2], o[3], 2});
         c.grid_tail = (int)std::max<long long>(std::min<long long>(std::max<long long>(slots / 4096, 8), most), a.n_stacks);
         if (most < a.n_stacks) c.grid_tail = 0;
         return r;
@@ -1716,7 +1719,9 @@ cudaError_t launch_tail(const Args &a, const GroupArgs &g, const GroupCfg &c, bo
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (g.tail_sums)
+    // a step by itself has little to add up: clearing and flushing took 1 us of the
+    // 66 of a call of one step and its window
+    if (g.tail_sums && g.end - g.off > 1)
         return det ? cudaLaunchKernelEx(&cfg, k_tail<true, true>, a, g) : cudaLaunchKernelEx(&cfg, k_tail<false, true>, a, g);
     return det ? cudaLaunchKernelEx(&cfg, k_tail<true, false>, a, g) : cudaLaunchKernelEx(&cfg, k_tail<false, false>, a, g);
 }
