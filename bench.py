@@ -144,23 +144,51 @@ def kernel_sha(name="pic_step.cuh"):
 # with their three comparisons for every carrier (14 per lane), about 250 per 32
 # eventful ones; issue slots per second from the SM count and the clock.
 WARP_INST_STEP, WARP_INST_EVENT = 14.0 / 32.0, 250.0 / 32.0
-# DRAM bytes per carrier-step of k_group's closed groups (the large bilayer scaled
-# to 1/20, 46 steps in a pass), valid for the source whose hash is given
-NCU_GROUP = {"bytes": 0.458, "src_sha": "2c885175345e7be5"}
+# DRAM bytes per carrier-step of k_group's closed groups without densities (the
+# large bilayer scaled to 1/20, 46 steps in a pass), valid for the source whose
+# hash is given.  It is what a pass moves over the steps of the pass, so it is
+# given for passes of about as many and no others.
+NCU_GROUP = {"bytes": 0.458, "steps": 46, "src_sha": "2c885175345e7be5"}
 
 
-def grouped_roofline(delta, k_ms, ms, time_steps, sms=152, sm_ghz=2.07):
+def device_rate():
+    """(SMs, maximum SM clock in GHz) of the device in use."""
+    import torch
+    sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+    try:
+        out = subprocess.run(["nvidia-smi", "--query-gpu=clocks.max.sm", "--format=csv,noheader,nounits"],
+                             capture_output=True, text=True, timeout=20).stdout
+        return sms, float(out.split()[0]) * 1e-3
+    except Exception:
+        return sms, 2.07
+
+
+def group_traffic(delta, ktimes, time_steps):
+    """DRAM bytes per time step of k_group, or None where the capture says
+    nothing: open groups (carriers created), densities inside the groups (every
+    pass counts as one with densities) or passes of other lengths."""
+    if delta["spawned"] or delta["injected"] or not ktimes["step"][0] or not ktimes["step_moments"][0]:
+        return None
+    steps = time_steps / ktimes["step_moments"][0]        # a pass ends at its window
+    if not 0.85 * NCU_GROUP["steps"] <= steps <= 1.15 * NCU_GROUP["steps"]:
+        return None
+    if NCU_GROUP["src_sha"] != kernel_sha("pic_group.cu"):
+        return None
+    return NCU_GROUP["bytes"] * delta["particle_steps"] / time_steps
+
+
+def grouped_roofline(delta, ktimes, k_ms, ms, time_steps):
+    sms, sm_ghz = device_rate()
     ps = delta["particle_steps"]
     need = (WARP_INST_STEP * ps + WARP_INST_EVENT * delta["eventful"]) / ps if ps else WARP_INST_STEP
     peak = sms * 4 * sm_ghz * 1e9 / need
     achieved = ps / (k_ms * 1e-3)
-    pinned = NCU_GROUP["bytes"] is not None and NCU_GROUP["src_sha"] == kernel_sha("pic_group.cu")
     return {"bound": "issue", "achieved": achieved, "peak": peak, "unit": "particle-steps/s",
             "frac": achieved / peak, "form": "grouped",
             "kernel": "k_group + k_tail (several time steps per pass over memory), k_dens",
             "peak_source": "%d SMs x 4 issue slots x %.2f GHz / %.2f warp instructions needed per "
                            "carrier-step" % (sms, sm_ghz, need),
-            "traffic": NCU_GROUP["bytes"] * ps / time_steps if pinned else None,
+            "traffic": group_traffic(delta, ktimes, time_steps),
             "avg_launch_ms": k_ms / time_steps,
             "kernel_share_of_step_time": k_ms / ms if ms else 0}
 
@@ -505,7 +533,7 @@ def roofline_of(delta, ktimes, ms, fused=False, time_steps=None):
     if not n_k or not k_ms:
         return None
     if time_steps and n_k < time_steps:
-        return grouped_roofline(delta, k_ms, ms, time_steps)
+        return grouped_roofline(delta, ktimes, k_ms, ms, time_steps)
     alg = B_STEP * delta["particle_steps"] + B_EVENTFUL * delta["eventful"] + \
         B_CHANGED * delta["changed"] + B_SPAWN * delta["spawned"]
     strict = S_STEP * delta["particle_steps"] + S_EVENTFUL * delta["eventful"] + \
