@@ -98,12 +98,13 @@ typedef struct {
                                cooperative launch (every block resident, the
                                passes of every step separated by grid barriers
                                with bounded waits), captured in a CUDA graph;
-                               grouped steps (event_pass 0) run each call of
-                               pic_step in one such launch; 0: one launch per
-                               kernel, or for grouped steps of up to 2^23 slots
-                               the single launch of 2.  Results are
-                               identical; kernel timing (pic_profile) always
-                               uses single launches. */
+                               what a call has besides whole periods is run as
+                               with 0; 0: one launch per kernel, or, for
+                               grouped steps (event_pass 0) without weights of
+                               up to 2^23 slots, all steps of a call that are
+                               more than a group in one persistent launch.
+                               Results are identical; kernel timing
+                               (pic_profile) always uses single launches. */
     int32_t stack_base;     /* global index of the context's first stack
                                (0..65535 - n_stacks): stack s draws the random
                                streams of stack stack_base + s, so that stacks
@@ -115,10 +116,17 @@ typedef struct {
                                consecutive slots of a 1024-slot tile); 0 = 8.
                                Results do not depend on it. */
     int32_t event_pass;     /* 0: the steps run in groups, several per pass over
-                               memory; where that does not fit (a moment grid
-                               of more than the shared memory, scattering
-                               probabilities within 2^-16 of 1), the ordinary
-                               steps of a single-stack context with eight
+                               memory, but for steps by themselves in larger
+                               contexts.  Where groups do not fit (a moment
+                               grid or tables that leave shared memory for
+                               fewer than 8 warps, or for the densities of one
+                               step only in a context of more than 2^21 slots;
+                               scattering probabilities within 2^-16 of 1;
+                               stacks thicker than 32768 nm; cells below
+                               1/1024 nm; more stacks than blocks that are
+                               resident at once), and for steps by
+                               themselves, the ordinary steps of a
+                               single-stack context with eight
                                consumer warps run the general step of the
                                eventful carriers inside the streaming pass
                                (extra warps fed through a shared-memory ring,
@@ -128,7 +136,10 @@ typedef struct {
                                depend on it. */
 } pic_params;
 
-/* Launch configuration a context chose (pic_launch_info). */
+/* Launch configuration a context chose for single steps (pic_launch_info):
+ * grouped steps, the default where they fit, have shapes of their own, and
+ * nothing here says whether a context's steps are grouped (pic_launch_count
+ * does: single steps take two launches each or more). */
 typedef struct {
     int32_t grid_step, grid_step_moments;   /* streaming pass */
     int32_t grid_slow, grid_slow_moments;   /* event pass */
@@ -140,8 +151,9 @@ typedef struct {
      * streaming pass with density weights, its ring depth and shared memory */
     int32_t grid_adj_step[2], ring_adj_step[2];
     int64_t smem_adj_step[2];
-    /* the streaming pass with the general step inside (event_pass 0); grid
-     * 0: ordinary steps use the separate event pass */
+    /* the streaming pass with the general step inside (event_pass 0), for
+     * ordinary steps that are not grouped; grid 0: these use the separate
+     * event pass */
     int32_t grid_step_fused, ring_step_fused;
     int64_t smem_step_fused;
 } pic_launch_info;
@@ -441,7 +453,9 @@ typedef struct {
     double ns_per_particle_step;  /* device time of the trial / carriers advanced */
     int32_t consumer_warps; /* warps of the streaming pass on the carriers (4 or 8),
                                i.e. 8 or 4 consecutive slots per thread */
-    int32_t event_pass;     /* 0 the general step inside the streaming pass, 1 separate */
+    int32_t event_pass;     /* 0 grouped steps (the other fields: the single steps between
+                               groups), or the general step inside the streaming pass
+                               where steps are not grouped; 1 a separate event pass */
 } pic_tune_entry;
 
 /* Time candidate launch configurations of the step kernels on the running
@@ -449,14 +463,15 @@ typedef struct {
  * trial_steps ordinary steps, grouped ones (event_pass 0) by at least a whole
  * group (results do not depend on the launch configuration: the slot order
  * and every random word are fixed by the run), timed with CUDA events on the
- * context stream and divided by the carriers advanced.  Candidates: grouped
- * steps, where the context can run them; single steps with 8 or 4 consumer
+ * context stream and divided by the carriers advanced.  Candidates: single
+ * steps with 8 or 4 consumer
  * warps per block of the streaming pass (4 or 8 slots per thread), 1 to 6 (8
  * with four warps) resident blocks per SM, ring depth 2, 3, 4, 6 or 8 where
- * it fits, both deposit modes when the trial contains density steps; and,
- * where steps cannot be grouped (eight consumer warps, a single stack), the
- * general step inside the streaming pass or in a separate pass.  entries (host, may be NULL): up to max_entries results in
- * the order tried; *n_entries (may be NULL): their number.  Needs steps left:
+ * it fits, both deposit modes when the trial contains density steps; where
+ * steps cannot be grouped (eight consumer warps, a single stack), the general
+ * step inside the streaming pass or in a separate pass; and grouped steps,
+ * where the context can run them, once and last.  entries (host, may be
+ * NULL): up to max_entries results in the order tried; *n_entries (may be NULL): their number.  Needs steps left:
  * up to 200 * trial_steps.  Synchronises. */
 pic_status pic_autotune(pic_ctx *ctx, int trial_steps, pic_tune_entry *entries,
                         int max_entries, int *n_entries);

@@ -220,7 +220,8 @@ struct Args {            // everything a kernel needs, passed by value
 // four in contexts of more than GROUP_LIST_SLOTS, where the new carriers, which
 // draw their test words one by one, would cost more than the passes over the others
 // save (500 steps from 2e7 carriers 85.0 against 86.5 ms with eight) and the record
-// lists of more steps would need memory of their own.
+// lists of more steps would need memory of their own (both sides measured before
+// the new carriers' sums went to shared memory).
 constexpr int GROUP_OPEN = 8, GROUP_OPEN_LARGE = 4;
 constexpr long long GROUP_LIST_SLOTS = 8ll << 20;
 // A step by itself (a call of one step, or densities so often and of so many bins

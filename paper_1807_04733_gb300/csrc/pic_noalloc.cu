@@ -67,7 +67,7 @@ extern "C" pic_status pic_compact_static(const float *z, const float *mu, const 
     if (n >= (int64_t(1) << 30)) return PIC_ERR_ARG;
     if (n > 0 && (!z || !mu || !id || !packed || !z_out || !mu_out || !id_out || !packed_out))
         return PIC_ERR_ARG;
-    // the kernel reads the inputs in 16-byte vectors
+    // (the interface asks for 16 bytes, whatever the kernel's loads need)
     if (n > 0 && ((reinterpret_cast<uintptr_t>(packed) | reinterpret_cast<uintptr_t>(z) |
                    reinterpret_cast<uintptr_t>(mu) | reinterpret_cast<uintptr_t>(id)) & 15u))
         return PIC_ERR_ARG;
