@@ -144,11 +144,12 @@ def kernel_sha(name="pic_step.cuh"):
 # with their three comparisons for every carrier (14 per lane), about 250 per 32
 # eventful ones; issue slots per second from the SM count and the clock.
 WARP_INST_STEP, WARP_INST_EVENT = 14.0 / 32.0, 250.0 / 32.0
-# DRAM bytes per carrier-step of k_group's closed groups without densities (the
-# large bilayer scaled to 1/20, 46 steps in a pass), valid for the source whose
-# hash is given.  It is what a pass moves over the steps of the pass, so it is
-# given for passes of about as many and no others.
-NCU_GROUP = {"bytes": 0.458, "steps": 46, "src_sha": "2c885175345e7be5"}
+# DRAM bytes per carrier-step of k_group over a period of 50 steps of a full buffer
+# without densities in the groups (the large bilayer scaled to 1/20: a pass of 4
+# steps after the compaction, 0.334 GB, and one of 46, 0.418 GB, for 1.0e9
+# carrier-steps), valid for the source whose hash is given.  It is what a pass
+# moves over the steps of the pass, so it is given for such periods and no others.
+NCU_GROUP = {"bytes": 0.751, "steps": 50, "src_sha": "42770416175d5ecf"}
 
 
 def device_rate():
@@ -165,12 +166,14 @@ def device_rate():
 
 def group_traffic(delta, ktimes, time_steps):
     """DRAM bytes per time step of k_group, or None where the capture says
-    nothing: open groups (carriers created), densities inside the groups (every
-    pass counts as one with densities) or passes of other lengths."""
-    if delta["spawned"] or delta["injected"] or not ktimes["step"][0] or not ktimes["step_moments"][0]:
+    nothing: carriers created in most steps, densities inside the groups (every
+    pass counts as one with densities) or periods of other lengths."""
+    if delta["spawned"] + delta["injected"] > 1e-4 * delta["particle_steps"]:
+        return None
+    if not ktimes["step"][0] or not ktimes["step_moments"][0]:
         return None
     steps = time_steps / ktimes["step_moments"][0]        # a pass ends at its window
-    if not 0.85 * NCU_GROUP["steps"] <= steps <= 1.15 * NCU_GROUP["steps"]:
+    if not 0.9 * NCU_GROUP["steps"] <= steps <= 1.1 * NCU_GROUP["steps"]:
         return None
     if NCU_GROUP["src_sha"] != kernel_sha("pic_group.cu"):
         return None
