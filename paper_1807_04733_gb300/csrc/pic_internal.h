@@ -167,11 +167,6 @@ struct Args {            // everything a kernel needs, passed by value
     uint32_t step;                           // time step (plain launches)
     const unsigned int *step_dev;            // graph replay: the step is read here
     int bump_step;                           // this kernel's last block advances *step_dev
-    // what is due at the end of a range of grouped steps runs only if the device
-    // step is due_step, in graphs (due_period > 0) whole periods after it; due 0:
-    // whatever it is
-    int due;
-    uint32_t due_step, due_period;
     int tab_max, T_max, nbin_max, jbin_max;  // shared-memory sizing
     int ftab_max;                            // entries of the padded fast table
     int gbin_max;                            // cells of the widest stack (generation sums)
@@ -212,6 +207,11 @@ struct Args {            // everything a kernel needs, passed by value
     // velocity moment [stack][n_out][2][n_cells] at n_off / n_e, units of
     // 2^-32 nm/fs (PIC_F_VELOCITY_MOMENTS)
     long long *v_hist;
+    // what is due at the end of a range of grouped steps runs only if the device
+    // step is due_step, in graphs (due_period > 0) whole periods after it; due 0:
+    // whatever it is
+    int due;
+    uint32_t due_step, due_period;
 };
 
 // Groups of time steps run in one pass over memory (pic_group.cu).
